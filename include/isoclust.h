@@ -79,7 +79,11 @@ enum {
 /* precision values: arithmetic of the Boruvka candidate sweep.  Every path
  * ends in the same FP64 key comparison, so all give the identical tree. */
 enum {
-    ISOCLUST_PREC_AUTO = 0,    /* F64 input: FP64 sweep; F32 input: tensor-core sweep    */
+    ISOCLUST_PREC_AUTO = 0,    /* sm_103: tensor-core sweep (F64 input: on an FP32 copy of
+                                  the centred, scaled points, keys from the points; the FP64
+                                  sweep when a spin limit is given or the largest magnitude
+                                  is outside 2^-500 .. 2^500); else F64 input: FP64 sweep,
+                                  F32 input: FP32 SIMT sweep                             */
     ISOCLUST_PREC_FP64 = 1,    /* FP64 sweep (exact keys directly)                       */
     ISOCLUST_PREC_FP32 = 2,    /* FP32 SIMT candidates, FP64 recheck in a proven margin  */
     ISOCLUST_PREC_BF16_TC = 3  /* BF16 hi+lo Gram tiles on tcgen05 tensor cores with FP32
@@ -105,7 +109,7 @@ typedef struct {
  * returns; the call then returns ISOCLUST_ERR_TIMEOUT without walking the
  * unfinished tree, and the device stays usable.  A small value can make
  * calls fail on a healthy device.  Calls without the tensor-core sweep
- * never wait. */
+ * never wait (F64 input with a spin_limit takes none). */
 
 /* Test hook of the timeout path (no paper counterpart): while on (1), the
  * epilogue of every tensor-core sweep launch first waits for a barrier that
@@ -446,7 +450,7 @@ double isoclust_last_omega_gram_ms(int64_t *blocks, int64_t *direct_pairs);
 isoclust_status isoclust_set_sweep_variant(int32_t variant);
 
 /* The sweep variant of the last minimum-spanning-tree build on this host
- * thread (0..3), or -1 when none ran (FP32/FP64 sweep, F64 input). */
+ * thread (0..3), or -1 when none ran (FP32/FP64 sweep). */
 int32_t isoclust_last_sweep_variant(void);
 
 /* How the last isoclust_cluster_batched / _batched_detail call on this

@@ -23,6 +23,9 @@ cudaError_t weights_launch_sym(const float *X, int64_t n, int32_t d, double sigm
                                cudaStream_t s, const Shard *sh = nullptr, double *part64 = nullptr,
                                OmegaGram *og = nullptr, uint32_t *status = nullptr, uint64_t wait_cycles = 0);
 float omega_zskip(int64_t n);
+size_t weights64_bytes(int64_t n, bool with_p);
+cudaError_t weights64_launch(const void *X, int64_t n, int32_t d, int dtype, double sigma, double alpha,
+                             int include_self, double *omega, double *p, void *part, cudaStream_t s);
 constexpr size_t SYM_PART_LIMIT = size_t(16) << 30;   // symmetric sweep up to 16 GiB of partials
 // the omega Gram goes to the tensor cores by default for rows at least this
 // long (measured on GB300: 1.23x faster at d = 64, 1.3x at d = 128, 5x at
@@ -196,11 +199,19 @@ namespace {
 constexpr int TPB = 256;
 
 template <class T>
-__global__ void k_check_finite(const T *__restrict__ X, int64_t count, uint32_t *st) {
+__global__ void k_check_finite(const T *__restrict__ X, int64_t count, uint32_t *st, unsigned long long *absmax) {
     bool bad = false;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
-        if (!isfinite((double)X[i])) bad = true;
+    unsigned long long m = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
+        const double x = (double)X[i];
+        if (!isfinite(x)) bad = true;
+        else if (absmax) m = max(m, (unsigned long long)dbits(fabs(x)));
+    }
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(st, DEV_NONFINITE);
+    if (absmax) {
+        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if ((threadIdx.x & 31) == 0 && m) atomicMax(absmax, m);
+    }
 }
 
 __global__ void k_tree_input(const int32_t *__restrict__ parent, int64_t n, int32_t *info, uint32_t *st) {
@@ -257,15 +268,15 @@ __global__ void k_scatter_rows(const double *__restrict__ vp, const int32_t *__r
 }
 }  // namespace
 
-cudaError_t check_finite(const void *X, int64_t count, int dtype, uint32_t *status, double *absmax, cudaStream_t s) {
-    (void)absmax;
+cudaError_t check_finite(const void *X, int64_t count, int dtype, uint32_t *status, unsigned long long *absmax,
+                         cudaStream_t s) {
     int64_t gb = ceil_div(count, TPB), gmax = (int64_t)num_sms() * 16;
     unsigned g = (unsigned)(gb < gmax ? gb : gmax);
     if (g == 0) g = 1;
     if (dtype == ISOCLUST_F64)
-        k_check_finite<double><<<g, TPB, 0, ISO_S(s)>>>((const double *)X, count, status);
+        k_check_finite<double><<<g, TPB, 0, ISO_S(s)>>>((const double *)X, count, status, absmax);
     else
-        k_check_finite<float><<<g, TPB, 0, ISO_S(s)>>>((const float *)X, count, status);
+        k_check_finite<float><<<g, TPB, 0, ISO_S(s)>>>((const float *)X, count, status, nullptr);
     return cudaGetLastError();
 }
 
@@ -424,7 +435,13 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     TcScratch TC;
     TC.wait_cycles = o.spin_limit;
     TC.stall_test = g_stall_test.load(std::memory_order_relaxed);
-    const int tsplits = use_tc ? tc_splits(n) : 1;
+    // F64 input with AUTO precision: the same sweep on an FP32 copy, keys from
+    // the points.  A caller's spin limit keeps the FP64 sweep, which never
+    // waits (such a call cannot run out of it).
+    TC.f64 = dtype == ISOCLUST_F64 && o.precision == ISOCLUST_PREC_AUTO && o.spin_limit == 0 && !TC.stall_test &&
+             tc_supported();
+    const bool tc_any = use_tc || TC.f64;
+    const int tsplits = tc_any ? tc_splits(n) : 1;
     if (sh) {
         // the sharded work: the tensor-core sweep and the symmetric omega sweep
         if (!use_tc || fp64_sweep || o.alpha != 0.0 || o.omega_mode != ISOCLUST_OMEGA_FULL || !need_labels ||
@@ -465,11 +482,15 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     const int gram_mode = g_omega_gram.load(std::memory_order_relaxed);
     const bool gram = symmetric && use_tc && ceil_div(n, 128) <= 65535 &&
                       (gram_mode == 1 || (gram_mode < 0 && d >= OMEGA_GRAM_MIN_D));
+    const bool weights64 = need_labels && dtype == ISOCLUST_F64 &&
+                           (o.omega_mode == ISOCLUST_OMEGA_FULL || o.alpha != 0.0) &&
+                           weights64_bytes(n, o.alpha != 0.0) <= SYM_PART_LIMIT;
     auto carve = [&](Arena &A, MstScratch &M, TreeScratch &TS, double **phi, double **om, double **pp, double **omtmp,
                      uint32_t **status) {
         *status = A.take<uint32_t>(4);
         M.carve(A, n, splits);
-        if (use_tc) TC.carve(A, n, d, tsplits_used, 0, 1, tlists);
+        if (tc_any) TC.carve(A, n, d, tsplits_used, 0, 1, tlists);
+        if (weights64) P.sym = (void *)A.take<unsigned char>(weights64_bytes(n, o.alpha != 0.0));
         if (need_labels) {
             TS.carve(A, n);
             *phi = A.take<double>(n);
@@ -512,15 +533,21 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     ev.rec(0, s);
     ISO_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t) * 4, s));
     if (need_labels) ISO_CUDA(cudaMemsetAsync(TS.status, 0, sizeof(uint32_t), s));
-    ISO_CUDA(check_finite(X, n * (int64_t)d, dtype, status, nullptr, s));
-    uint32_t hst = 0;
-    ISO_CUDA(cudaMemcpyAsync(&hst, status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    // (status words 2 and 3: the largest magnitude, F64 input)
+    ISO_CUDA(check_finite(X, n * (int64_t)d, dtype, status, TC.f64 ? (unsigned long long *)(status + 2) : nullptr, s));
+    struct { uint32_t st, pad; double absmax; } hv = {0, 0, 0.0};
+    ISO_CUDA(cudaMemcpyAsync(&hv, status, sizeof(hv), cudaMemcpyDeviceToHost, s));
     ISO_CUDA(cudaStreamSynchronize(s));
-    if (hst) return map_status(hst, false);
+    if (hv.st) return map_status(hv.st, false);
     ev.rec(1, s);
+    bool tc_used = use_tc;
+    if (TC.f64 && hv.absmax > TC64_ABS_MIN && hv.absmax < TC64_ABS_MAX) {
+        tc_used = true;
+        frexp(hv.absmax, &TC.scale_exp);                // scaled points below 1
+    }
 
     // Section 2.2 steps 1-2: minimum spanning tree
-    ISO_CUDA(mst_build(M, X, n, d, dtype, fp64_sweep, status, s, use_tc ? &TC : nullptr, 1, 0, sh));
+    ISO_CUDA(mst_build(M, X, n, d, dtype, fp64_sweep, status, s, tc_used ? &TC : nullptr, 1, 0, sh));
     const bool mst_pruned = TC.prune && TC.prune_ready;     // (the omega screen re-prepares TC later)
     unsigned long long mst_swept = 0;
     if (mst_pruned) {
@@ -588,6 +615,8 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
                     ISO_CUDA(cudaMemsetAsync(pp, 0, sizeof(double) * n, s));
                 else
                     k_scatter_rows<<<gb, TPB, 0, ISO_S(s)>>>(P.pp, P.perm, n, pp);
+            } else if (weights64) {
+                ISO_CUDA(weights64_launch(X, n, d, dtype, sigma, o.alpha, o.include_self, om_out, pp, P.sym, s));
             } else {
                 ISO_CUDA(weights_launch(X, n, d, dtype, false, sigma, o.alpha, o.include_self, M.nnbits, om_out, pp,
                                         nullptr, s));
@@ -633,7 +662,7 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     g_prof_cnt[2] = ss.passes + (need_labels ? 1 : 0);
     g_prof_cnt[3] = ss.max_depth;
     g_prof_mst_tiles[0] = g_prof_mst_tiles[1] = 0;
-    if (use_tc) {
+    if (tc_used) {
         const int64_t nt = TC.n_pad / 128;
         g_prof_mst_tiles[1] = (int64_t)cnt[MC_ROUNDS] * nt * nt;
         g_prof_mst_tiles[0] = g_prof_mst_tiles[1];
@@ -1258,6 +1287,9 @@ isoclust_status isoclust_vertex_weights(const void *X, int64_t n, int32_t d, int
     TC.wait_cycles = o.spin_limit;
     TC.stall_test = g_stall_test.load(std::memory_order_relaxed);
     const int tsplits = use_tc ? tc_splits(n) : 1;
+    const size_t w64 = fp64 ? weights64_bytes(n, o.alpha != 0.0 && p) : 0;
+    const bool sym64 = fp64 && w64 <= SYM_PART_LIMIT;
+    void *part64 = nullptr;
     const int dev = current_device();
     std::lock_guard<std::mutex> lock(g_call_mu[dev]);
     MstScratch M;
@@ -1266,12 +1298,14 @@ isoclust_status isoclust_vertex_weights(const void *X, int64_t n, int32_t d, int
     status = meas.take<uint32_t>(4);
     M.carve(meas, n, splits);
     if (use_tc) TC.carve(meas, n, d, tsplits);
+    if (sym64) meas.take<unsigned char>(w64);
     void *base = scratch_acquire(meas.off, s, &st);
     if (!base) return st;
     Arena A{(char *)base, meas.off + 4096, 0, false};
     status = A.take<uint32_t>(4);
     M.carve(A, n, splits);
     if (use_tc) TC.carve(A, n, d, tsplits);
+    if (sym64) part64 = (void *)A.take<unsigned char>(w64);
     ISO_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t) * 4, s));
     ISO_CUDA(check_finite(X, n * (int64_t)d, dtype, status, nullptr, s));
     uint32_t hst = 0;
@@ -1279,7 +1313,10 @@ isoclust_status isoclust_vertex_weights(const void *X, int64_t n, int32_t d, int
     ISO_CUDA(cudaStreamSynchronize(s));
     if (hst) return map_status(hst, false);
     if (!fp64) ISO_CUDA(nn_sweep(M, X, n, d, dtype, fp64, status, s, use_tc ? &TC : nullptr));
-    ISO_CUDA(weights_launch(X, n, d, dtype, fp64, sigma, o.alpha, o.include_self, M.nnbits, omega, p, nullptr, s));
+    if (sym64)
+        ISO_CUDA(weights64_launch(X, n, d, dtype, sigma, o.alpha, o.include_self, omega, p, part64, s));
+    else
+        ISO_CUDA(weights_launch(X, n, d, dtype, fp64, sigma, o.alpha, o.include_self, M.nnbits, omega, p, nullptr, s));
     ISO_CUDA(cudaStreamSynchronize(s));
     ISO_CUDA(cudaMemcpy(&hst, status, sizeof(uint32_t), cudaMemcpyDeviceToHost));
     return map_status(hst, false);

@@ -134,9 +134,10 @@ cudaError_t exclusive_scan_i64(const int64_t *in, int64_t *out, int64_t n, int64
 cudaError_t sort_pairs_u64(uint64_t *keys, int32_t *vals, uint64_t *kbuf, int32_t *vbuf,
                            int64_t n, cudaStream_t s);
 
-// Non-finite scan of an input array (validation.cu): ORs DEV_NONFINITE.
+// Non-finite scan of an input array: ORs DEV_NONFINITE.  absmax (may be null,
+// F64 only, zero before): bits of the largest magnitude of the finite values.
 cudaError_t check_finite(const void *X, int64_t count, int dtype, uint32_t *status,
-                         double *absmax, cudaStream_t s);
+                         unsigned long long *absmax, cudaStream_t s);
 
 // ---------------------------------------------------------------- device helpers
 __device__ __forceinline__ uint64_t dbits(double x) { return (uint64_t)__double_as_longlong(x); }

@@ -68,6 +68,14 @@ struct TcScratch {
     // and the first padded row of each set (device arrays)
     const int4 *items = nullptr;
     int64_t nitems = 0;
+    // FP64 input: the sweep, its bounds and the FP32 filter run on xf, the
+    // points less their mean, times a power of two, rounded to FP32; keys
+    // are taken from x64, the points themselves
+    bool f64 = false;
+    const double *x64 = nullptr;
+    float *xf = nullptr;                           // [n][d]
+    double *mean64 = nullptr;
+    int scale_exp = 0;                             // the power of two is 2^-scale_exp
     int32_t nsets = 1;
     const int32_t *set_of = nullptr;
     const int64_t *offs = nullptr;
@@ -121,6 +129,8 @@ bool tc_supported();
 // place = false: the rows are placed later (tc_place_rows, by the pruned
 // rounds' order); only the mean, maps and buffers are prepared.
 cudaError_t tc_prepare(TcScratch &T, const float *X, int64_t n, int32_t d, cudaStream_t s, bool place = true);
+// FP64 input: T.xf from T.x64 (centred, scaled by 2^-T.scale_exp).
+cudaError_t tc_rows_from_f64(TcScratch &T, int64_t n, int32_t d, cudaStream_t s);
 cudaError_t tc_sweep_round(TcScratch &T, MstScratch &S, const float *X, int64_t n, int32_t d, uint32_t *status,
                            cudaStream_t s);
 // omega screen on the tensor cores: Xp (n x d, omega's row order) and its
@@ -142,8 +152,12 @@ void tc_clear_last_variant();           // a build without the tensor-core sweep
 // independent sets: recount the components of every set from comp
 cudaError_t tc_count_sets(TcScratch &T, const int32_t *comp, int64_t n, const int32_t *counters, cudaStream_t s);
 
+// FP64 points whose largest magnitude is outside this range keep the FP64
+// sweep: scaled squares stay clear of FP32's and FP64's exponent limits.
+constexpr double TC64_ABS_MIN = 0x1p-500, TC64_ABS_MAX = 0x1p500;
+
 // Builds the MST of X (n x d, dtype F32/F64) into S.eu/ev/ed2 (unsorted).
-// tc != nullptr selects the tensor-core sweep (F32 input).
+// tc != nullptr selects the tensor-core sweep (F32 input, or F64 with tc->f64).
 // sweep_fp64: use the exact FP64 sweep instead of FP32 + recheck.
 // rounds_out / rescans_out: host copies of the round and rescan counts are
 // written after the final stream synchronisation by the caller.

@@ -22,6 +22,7 @@
 // The candidates are exact-keyed in FP64 by k_recheck_tc inside a rigorous
 // error margin; rows whose margin is not closed by the best 8 are rescanned.
 #include <cuda.h>
+#include <math.h>
 #include <stddef.h>
 
 #include <atomic>
@@ -802,6 +803,15 @@ __device__ __forceinline__ void rc_dist(const float *__restrict__ xs, int64_t r,
     }
 }
 
+// FP64 input: the FP32 copy of a point is off by at most eps64 times its norm
+// (its rounding, 2^-24 per coordinate), so two points' distance moves by at
+// most w, and a column that holds the exact best has an FP32 distance within
+// 2 w of the bound without that error.
+__device__ __forceinline__ float widen_f64(float thr, float w) {
+    const float a = __fadd_ru(__fsqrt_ru(thr), __fadd_ru(w, w));
+    return __fmul_ru(__fmul_ru(a, a), 1.00001f);
+}
+
 template <int EPL, int CW>
 __device__ __forceinline__ void recheck_row(int64_t r, int lane, const float *__restrict__ xs, int64_t n, int32_t d,
                                             int lists, const float *__restrict__ tv, const int32_t *__restrict__ tj,
@@ -813,7 +823,7 @@ __device__ __forceinline__ void recheck_row(int64_t r, int lane, const float *__
                                             const int32_t *__restrict__ set_of, const int32_t *__restrict__ setcnt,
                                             int32_t *counters, int32_t *__restrict__ bj_s, int shard_rank,
                                             int shard_world,
-                                            const int32_t *__restrict__ row_lists) {
+                                            const int32_t *__restrict__ row_lists, float eps64) {
     if (lane == 0) nsurv[r] = 0;           // every row, padding included: k_exact_tc reads them all
     const int64_t i = perm[r];
     if (i < 0) return;                     // padding row
@@ -943,7 +953,8 @@ __device__ __forceinline__ void recheck_row(int64_t r, int lane, const float *__
         if (lane == 0) rowj[i] = -1;
         return;
     }
-    const float thr = __fadd_ru(__fmul_ru(m32, mul32), add32);
+    float thr = __fadd_ru(__fmul_ru(m32, mul32), add32);
+    if (eps64 > 0.0f) thr = widen_f64(thr, __fmul_ru(eps64, __fadd_ru(si, smax)));
     int ns = 0;
 #pragma unroll
     for (int p = 0; p < NPASS; ++p) {
@@ -983,7 +994,10 @@ __device__ __forceinline__ void recheck_row(int64_t r, int lane, const float *__
 
 // Exact keys of the recorded columns, one thread per row: the FP64 pipe sees
 // full warps (a warp per row would run each key on a single lane).
-__global__ void __launch_bounds__(256) k_exact_tc(const float *__restrict__ xs, int64_t n, int32_t d,
+// x: the rows in the sweep's order (FP32 input, by_point 0) or the FP64 points
+// themselves (by_point 1: row perm[r]).
+template <class P>
+__global__ void __launch_bounds__(256) k_exact_tc(const P *__restrict__ x, int by_point, int64_t n, int32_t d,
                                                   const int32_t *__restrict__ perm, const int32_t *__restrict__ nsurv,
                                                   const int32_t *__restrict__ surv, double *__restrict__ rowd2,
                                                   int32_t *__restrict__ rowj, const int32_t *counters) {
@@ -993,7 +1007,7 @@ __global__ void __launch_bounds__(256) k_exact_tc(const float *__restrict__ xs, 
         const int c = nsurv[r];
         const int32_t i = perm[r];
         if (c <= 0 || c > TC_SURV || i < 0) continue;
-        const float *xi = xs + r * d;
+        const P *xi = x + (by_point ? (int64_t)i : r) * d;
         double best = INFINITY;
         int32_t bestj = -1;
         for (int q = 0; q < c; ++q) {
@@ -1001,7 +1015,7 @@ __global__ void __launch_bounds__(256) k_exact_tc(const float *__restrict__ xs, 
             if (jp < 0 || jp >= n) continue;
             const int32_t j = perm[jp];
             if (j < 0) continue;
-            const double e = exact_d2(xi, xs + jp * d, d);
+            const double e = exact_d2(xi, x + (by_point ? (int64_t)j : jp) * d, d);
             if (bestj < 0 || key_less(e, i, j, best, i, bestj)) {
                 best = e;
                 bestj = j;
@@ -1024,7 +1038,7 @@ __global__ void __launch_bounds__(256, 4) k_recheck_tc(const float *__restrict__
                                                        int32_t *__restrict__ ovf, const int32_t *__restrict__ set_of,
                                                        const int32_t *__restrict__ setcnt, int32_t *counters,
                                                        int shard_rank, int shard_world,
-                                                       const int32_t *__restrict__ row_lists) {
+                                                       const int32_t *__restrict__ row_lists, float eps64) {
     if (!mst_active(counters)) return;
     __shared__ int32_t bj_s[8][TC_TOPK];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -1033,17 +1047,22 @@ __global__ void __launch_bounds__(256, 4) k_recheck_tc(const float *__restrict__
     for (int64_t r = w0; r < n; r += nw)
         recheck_row<EPL, CW>(r, lane, xs, n, d, lists, tv, tj, tu, rsq, perm, compp, nmax_bits, eps_rep, mul32, add32, nsurv,
                              surv, rowj, ovf, set_of, setcnt, counters, bj_s[wib], shard_rank,
-                             shard_world, row_lists);
+                             shard_world, row_lists, eps64);
 }
 
 // Self-contained rescan of a queued row: FP32 direct differences give the
 // minimum m; every column within the FP32 error margin of m is keyed in FP64.
 // With independent sets only the row's own set is scanned.
-__global__ void __launch_bounds__(256) k_rescan_tc(const float *__restrict__ X, int64_t n, int32_t d,
+// Xe: the points the keys are taken from (FP64 input: X is their FP32 copy).
+template <class P>
+__global__ void __launch_bounds__(256) k_rescan_tc(const float *__restrict__ X, const P *__restrict__ Xe, int64_t n,
+                                                   int32_t d,
                                                    const int32_t *__restrict__ comp, const int32_t *__restrict__ ovf,
                                                    const int32_t *__restrict__ set_of, const int64_t *__restrict__ offs,
-                                                   double mul, double add, double *__restrict__ rowd2,
-                                                   int32_t *__restrict__ rowj, int32_t *counters) {
+                                                   double mul, double add, float eps64,
+                                                   const unsigned int *__restrict__ nmax_bits,
+                                                   double *__restrict__ rowd2, int32_t *__restrict__ rowj,
+                                                   int32_t *counters) {
     if (!mst_active(counters)) return;
     __shared__ float smin[256];
     __shared__ double sd[256];
@@ -1070,7 +1089,11 @@ __global__ void __launch_bounds__(256) k_rescan_tc(const float *__restrict__ X, 
             if (threadIdx.x < s) smin[threadIdx.x] = fminf(smin[threadIdx.x], smin[threadIdx.x + s]);
             __syncthreads();
         }
-        const double tau = (double)smin[0] * mul + add;
+        double tau = (double)smin[0] * mul + add;
+        if (eps64 > 0.0f) {                       // (see widen_f64; |y_i| <= |y_max|)
+            const double a = sqrt(tau) + 4.0 * (double)eps64 * sqrt((double)__uint_as_float(*nmax_bits));
+            tau = a * a * (1.0 + 1e-6);
+        }
         double bd = INFINITY;
         int32_t bjj = -1;
         for (int64_t j = j0 + threadIdx.x; j < j1; j += 256) {
@@ -1081,7 +1104,7 @@ __global__ void __launch_bounds__(256) k_rescan_tc(const float *__restrict__ X, 
                 acc = __fmaf_rn(df, df, acc);
             }
             if ((double)acc <= tau) {
-                const double e = exact_d2(xi, X + j * d, d);
+                const double e = exact_d2(Xe + i * d, Xe + j * d, d);
                 if (bjj < 0 || key_less(e, (int32_t)i, (int32_t)j, bd, (int32_t)i, bjj)) { bd = e; bjj = (int32_t)j; }
             }
         }
@@ -1186,6 +1209,10 @@ void TcScratch::carve(Arena &A, int64_t n, int32_t d, int splits_, int64_t n_pad
     tu = A.take<float>((size_t)lists * n_pad);
     err = A.take<uint32_t>(4);
     qctr = A.take<uint32_t>(4);
+    if (f64) {
+        xf = A.take<float>((size_t)n * d, 256);
+        mean64 = A.take<double>(d);
+    }
     setcnt = nmeans > 1 || n_pad_rows > 0 ? A.take<int32_t>((size_t)(nmeans > 0 ? nmeans : 1)) : nullptr;
     if (prune) {
         tcen = A.take<float>((size_t)nt * d);
@@ -1448,6 +1475,58 @@ cudaError_t tc_prepare(TcScratch &T, const float *X, int64_t n, int32_t d, cudaS
     return cudaGetLastError();
 }
 
+// part [64][d], then the mean, of the points times sc (a power of two)
+__global__ void __launch_bounds__(256) k_f64_mean_partial(const double *__restrict__ X, int64_t n, int32_t d, double sc,
+                                                          int64_t rows_per, double *__restrict__ part) {
+    __shared__ double acc[8][33];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const int t = blockIdx.y * 32 + lane;
+    const int64_t r0 = (int64_t)blockIdx.x * rows_per, r1 = min(n, r0 + rows_per);
+    double s = 0.0;
+    if (t < d)
+        for (int64_t r = r0 + wp; r < r1; r += 8) s += X[r * d + t] * sc;
+    acc[wp][lane] = s;
+    __syncthreads();
+    if (wp == 0 && t < d) {
+        double sum = 0.0;
+        for (int w = 0; w < 8; ++w) sum += acc[w][lane];
+        part[(int64_t)blockIdx.x * d + t] = sum;
+    }
+}
+
+__global__ void k_f64_mean_final(const double *__restrict__ part, int nparts, int64_t n, int32_t d,
+                                 double *__restrict__ mean) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= d) return;
+    double s = 0.0;
+    for (int p = 0; p < nparts; ++p) s += part[(int64_t)p * d + t];
+    mean[t] = s / (double)n;
+}
+
+__global__ void k_f64_rows(const double *__restrict__ X, const double *__restrict__ mean, double sc, int64_t n,
+                           int32_t d, float *__restrict__ xf) {
+    const int64_t gs = (int64_t)gridDim.x * blockDim.x, tot = n * (int64_t)d;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += gs)
+        xf[e] = (float)__dsub_rn(X[e] * sc, mean[(int32_t)(e % d)]);
+}
+
+// FP64 points through the BF16 sweep: its bounds only have to hold for the
+// points, and one more rounding (2^-24 of a coordinate, when the centred
+// points become FP32) fits in the headroom of the BF16 split's 2^-18; the
+// FP32 filter's cut widens by it (widen_f64) and the keys come from the FP64
+// points, so the tree is the same bit for bit.  The FP64 sweep it replaces
+// does 3 d operations per ordered pair and round on a pipe of 2 per clock and
+// SM: 20,011 x 24 took 591 ms against 1.9, 2,000 x 8 21.5 ms against 0.59.
+cudaError_t tc_rows_from_f64(TcScratch &T, int64_t n, int32_t d, cudaStream_t s) {
+    const double sc = ldexp(1.0, -T.scale_exp);
+    k_f64_mean_partial<<<dim3(64, (unsigned)ceil_div(d, 32)), 256, 0, ISO_S(s)>>>(T.x64, n, d, sc, ceil_div(n, 64),
+                                                                                 T.part);
+    k_f64_mean_final<<<(unsigned)ceil_div(d, 128), 128, 0, ISO_S(s)>>>(T.part, 64, n, d, T.mean64);
+    const int64_t b = ceil_div(n * (int64_t)d, 256), cap = (int64_t)num_sms() * 16;
+    k_f64_rows<<<(unsigned)(b < cap ? b : cap), 256, 0, ISO_S(s)>>>(T.x64, T.mean64, sc, n, d, T.xf);
+    return cudaGetLastError();
+}
+
 cudaError_t tc_place_rows(TcScratch &T, const float *X, int64_t n, int32_t d, cudaStream_t s) {
     cudaError_t e;
     if ((e = cudaMemsetAsync(T.permp, 0xff, sizeof(int32_t) * T.n_pad, s))) return e;     // -1: padding
@@ -1528,6 +1607,9 @@ cudaError_t tc_sweep_round(TcScratch &T, MstScratch &S, const float *X, int64_t 
     const double e = 1.1 * (double)(d + 3) * 5.9604644775390625e-08;
     const double mul = (1.0 + e) / (1.0 - e);
     const double add = (double)(d + 1) * 1.401298464324817e-45 * 4.0;
+    // FP64 input: one rounding per coordinate of the FP32 copy, 25 % headroom
+    // (which also covers the copy's own mean not being exactly zero)
+    const float eps64 = T.f64 ? (float)(1.25 * 5.9604644775390625e-08) : 0.0f;
     const float mul32 = (float)(mul * (1.0 + 1e-6)), add32 = (float)(2.01 * add) + 1.401298464324817e-45f;
     const int64_t rblocks = ceil_div(T.n_pad * 32, 256), rcap = (int64_t)num_sms() * 16;
     // entries per lane of the list merge: lists x 8 <= 32 EPL (lists <= 32)
@@ -1535,7 +1617,7 @@ cudaError_t tc_sweep_round(TcScratch &T, MstScratch &S, const float *X, int64_t 
     k_recheck_tc<EPLV, CWV><<<(unsigned)(rblocks < rcap ? rblocks : rcap), 256, 0, ISO_S(s)>>>(                        \
         T.xs, T.n_pad, d, T.lists, T.tv, T.tj, T.tu, T.rsq, T.permp, T.compp, T.nmax_bits, (float)(eps_rep * 1.0001),  \
         mul32, add32, T.nsurv, T.surv, S.rowj, S.ovf_rows, T.set_of, T.setcnt, S.counters, T.shard_rank,           \
-        T.shard_world, pruned ? T.nlists : nullptr)
+        T.shard_world, pruned ? T.nlists : nullptr, eps64)
     if (T.lists <= 4)
         {
         if (T.cw == 32) ISO_RECHECK_LAUNCH(1, 32);
@@ -1558,11 +1640,20 @@ cudaError_t tc_sweep_round(TcScratch &T, MstScratch &S, const float *X, int64_t 
     }
 #undef ISO_RECHECK_LAUNCH
     const int64_t xblocks = ceil_div(T.n_pad, 256), xcap = (int64_t)num_sms() * 8;
-    k_exact_tc<<<(unsigned)(xblocks < xcap ? xblocks : xcap), 256, 0, ISO_S(s)>>>(T.xs, T.n_pad, d, T.permp, T.nsurv,
-                                                                                  T.surv, S.rowd2, S.rowj,
-                                                                                  S.counters);
-    k_rescan_tc<<<(unsigned)(num_sms() * 4), 256, 0, ISO_S(s)>>>(X, n, d, S.comp, S.ovf_rows, T.set_of, T.offs, mul,
-                                                                 add, S.rowd2, S.rowj, S.counters);
+    const unsigned xg = (unsigned)(xblocks < xcap ? xblocks : xcap);
+    if (T.f64) {
+        k_exact_tc<double><<<xg, 256, 0, ISO_S(s)>>>(T.x64, 1, T.n_pad, d, T.permp, T.nsurv, T.surv, S.rowd2, S.rowj,
+                                                     S.counters);
+        k_rescan_tc<double><<<(unsigned)(num_sms() * 4), 256, 0, ISO_S(s)>>>(
+            X, T.x64, n, d, S.comp, S.ovf_rows, T.set_of, T.offs, mul, add, eps64, T.nmax_bits, S.rowd2, S.rowj,
+            S.counters);
+    } else {
+        k_exact_tc<float><<<xg, 256, 0, ISO_S(s)>>>(T.xs, 0, T.n_pad, d, T.permp, T.nsurv, T.surv, S.rowd2, S.rowj,
+                                                    S.counters);
+        k_rescan_tc<float><<<(unsigned)(num_sms() * 4), 256, 0, ISO_S(s)>>>(
+            X, X, n, d, S.comp, S.ovf_rows, T.set_of, T.offs, mul, add, 0.0f, T.nmax_bits, S.rowd2, S.rowj,
+            S.counters);
+    }
     (void)status;
     return cudaGetLastError();
 }

@@ -16,7 +16,9 @@
 // range; omega_i = exp(-y_i,nn) * sum is formed in FP64 at the end.
 // Rows are owned by threads (4x4 pairs per thread, 64x64 tiles), so each
 // row's sum has a fixed order: the result is deterministic.
-// FP64 input uses a plain FP64 kernel with the reference summation order.
+// FP64 input takes the symmetric FP64 kernel of weights64.cu; the plain one
+// here serves only sizes whose partial sums would pass that kernel's memory
+// limit (about 260,000 points).
 #include <math.h>
 
 #include "common.cuh"
@@ -1079,7 +1081,8 @@ __global__ void k_weights_reduce_sets(const unsigned long long *__restrict__ nnb
     omega[r] = w2;
 }
 
-// FP64 input: canonical FP64 terms, j ascending (the oracle's order).
+// FP64 terms, one thread per row, j ascending: only past weights64.cu's memory
+// limit.
 template <class T>
 __global__ void __launch_bounds__(TPB) k_weights_f64(const T *__restrict__ X, int64_t n, int32_t d, double sigma,
                                                      double alpha, int include_self, double *__restrict__ omega,
