@@ -216,7 +216,7 @@ def omega_roofline(torch, dev, prof, n_pairs_alg, d, workload, sets=False):
     tiles, tiles_dw, sym = prof[-1]["omega_tiles"], prof[-1]["omega_tiles_dw"], prof[-1]["omega_symmetric"]
     alg_flop = n_pairs_alg * (2.0 * d + 25.0)
     if sym == 3:
-        return omega_gram_roofline(prof, peaks, src, alu_peak, sms, w_ms, tiles_dw, d, alg_flop)
+        return omega_fused_roofline(prof, peaks, src, alu_peak, sms, w_ms, tiles_dw, d, alg_flop)
     screen_ops = 0.0 if (sym == 2 or sets) else 2.0 * d + (12.0 if sym else 8.0)
     dw_ops = (18.75 * d + 95.0) if (sym or sets) else (21.0 * d + 75.0)
     work = tiles * 4096.0 * screen_ops + tiles_dw * 4096.0 * dw_ops
@@ -242,8 +242,40 @@ def omega_roofline(torch, dev, prof, n_pairs_alg, d, workload, sets=False):
     }
 
 
+def omega_fused_roofline(prof, peaks, src, alu_peak, sms, kernel_ms, items, d, alg_flop):
+    """omega with the Gram on the tensor cores, one kernel: ALU-bound for rows
+    of up to about 1,000 dimensions, tensor-bound beyond.  FP32-pipe
+    instructions of the algorithm as built: 147 per pair of a kept 64 x 64
+    tile pair (fold of the accumulators 28, d2 and its test 27, root 12, shift
+    15, double-word exp 48, the two sums 17) and 18.75 d + 95 per pair that took
+    the direct sum; MMAs as issued: 34 digit-plane products of
+    2 x 128 x 64 x d_pad flop per 128 x 64 block.  The line reports the larger
+    fraction."""
+    blocks, direct = prof[-1]["omega_gram_blocks"], prof[-1].get("omega_gram_direct_pairs", 0)
+    seconds = kernel_ms / 1000.0
+    bf16 = peaks.get("bf16_tflops", 1900.0)
+    tc = blocks * 34 * 2.0 * 128 * 64 * (-(-d // 16) * 16) / seconds / 1e12
+    alu = (items * 4096.0 * 147.0 + direct * (18.75 * d + 95.0)) / seconds / 1e12
+    alg = alg_flop / seconds / 1e12
+    tensor = {"bound": "tensor", "achieved": tc, "peak": bf16, "frac": tc / bf16, "blocks": blocks}
+    vector = {"bound": "alu", "achieved": alu, "peak": alu_peak, "frac": alu / alu_peak, "direct_pairs": direct,
+              "direct_share": direct / max(1.0, items * 4096.0)}
+    top, other = (tensor, vector) if tc / bf16 > alu / alu_peak else (vector, tensor)
+    return dict(top, unit="TFLOP/s", kernel="k_omega_tc (omega, Gram on tcgen05 and double-word FP32 terms)",
+                kernel_ms=kernel_ms, traffic=None, other_unit=other,
+                note=f"FP32-pipe instructions of the algorithm as built (147 per pair of the {items} kept 64x64 tile "
+                     f"pairs, 18.75 d + 95 per direct pair) over {sms} SMs x {FP32_LANES_PER_SM} lanes x max SM clock "
+                     f"({src} sm_max_mhz), and the digit-plane MMAs over the measured BF16 peak, both over the "
+                     f"kernel's CUDA-event time ({kernel_ms:.2f} ms)",
+                algorithmic={"achieved": alg, "unit": "FP64-equivalent TFLOP/s", "peak": None,
+                             "flop_per_launch": alg_flop,
+                             "note": "the method's work (eq. omega over all pairs, (2d + 25) FP64-equivalent flop each) "
+                                     "over the kernel's time; no measured peak exists in this unit"})
+
+
 def omega_gram_roofline(prof, peaks, src, alu_peak, sms, sweep_ms, items, d, alg_flop):
-    """omega with the Gram on the tensor cores: two kernels.  The Gram kernel
+    """omega with the Gram on the tensor cores as two kernels, the form that
+    the captures at 40,000 x 64 were taken of.  The Gram kernel
     (tensor-bound: 34 BF16 digit-plane products of 2 x 128 x 64 x d_pad
     flop per 128 x 64 block, executed) and the sweep that reads it
     (ALU-bound, FP32-pipe instructions of the algorithm as built: per pair of

@@ -422,15 +422,14 @@ void isoclust_last_omega_tiles(int64_t *tiles3);
 /* Device time (milliseconds, CUDA events on the call's stream around its
  * launch) of the dominant pair kernel of the last call on this host thread:
  * the symmetric omega kernel after isoclust_cluster / _detail / _batched (0
- * when it did not run; with the Gram on the tensor cores, the sweep that
- * reads it), the pair-sum kernel of dOmega after isoclust_ik_backward. */
+ * when it did not run), the pair-sum kernel of dOmega after isoclust_ik_backward. */
 double isoclust_last_omega_kernel_ms(void);
 
-/* Device time (milliseconds, CUDA events on the call's stream) of the
- * tensor-core Gram kernel of omega in the last one-set call on this host
+/* Device time (milliseconds, CUDA events on the call's stream) of the omega
+ * kernel with the Gram on the tensor cores in the last call on this host
  * thread (isoclust_set_omega_gram), 0 when it did not run; *blocks (may be
  * NULL) gets its number of 128 x 64 blocks (each 34 BF16 digit-plane MMA
- * products of 2 x 128 x 64 x d_pad flop, d_pad = d rounded up to 64), and
+ * products of 2 x 128 x 64 x d_pad flop, d_pad = d rounded up to 16), and
  * *direct_pairs (may be NULL) the number of pairs whose Gram form cancelled
  * and which took the direct sum of squared differences instead. */
 double isoclust_last_omega_gram_ms(int64_t *blocks, int64_t *direct_pairs);
@@ -462,21 +461,21 @@ int32_t isoclust_last_sweep_variant(void);
  * captured).  Results are identical in every mode. */
 int32_t isoclust_last_batched_graph_mode(void);
 
-/* Arithmetic of eq. omega's pair sums in one-set calls (F32 input, sm_103,
- * alpha = 0, full-graph omega).  Tensor-core Gram: each kept tile pair's
- * Gram <y_i, y_j> of the tile-centred points is formed exactly on the tensor
- * cores (7 balanced base-256 digit planes per row, BF16 products summed
- * exactly in FP32 accumulators), the rest of d2 and the terms in double-word
- * FP32, and pairs whose Gram form cancels (its parts more than twice d2)
- * take the double-word sum of squared differences.  Otherwise every pair's
- * d2 is that double-word sum.  Both keep d2 to about 2^-46 relative; omega
- * agrees to within the library's error bound, not bit for bit.
- * Rows of 1,024 dimensions or more are centred on one point for the Gram
- * (the mean of the 64-row tiles' centroids), shorter ones on their tile's
- * centroid.
- * mode -1 (the default): the Gram on the tensor cores for rows of 64
- * dimensions or more; 1: always; 0: never.  Process-wide; other values ->
- * INVALID_ARG. */
+/* Arithmetic of eq. omega's pair sums (F32 input, sm_103, alpha = 0,
+ * full-graph omega; one set, and independent sets).  Tensor-core Gram: each
+ * kept tile pair's Gram <y_i, y_j> of the centred points is formed on the
+ * tensor cores from 7 balanced base-256 digit planes per row (BF16 products,
+ * exact FP32 sums of the leading weights), the rest of d2 and the terms in
+ * double-word FP32 by the same kernel, and pairs whose Gram form cancels (its
+ * parts more than 4 times d2, twice for rows far from all others) take the
+ * double-word sum of squared differences.  Otherwise every pair's d2 is that
+ * double-word sum.  Both keep d2 to about 2^-46 relative; omega agrees to
+ * within the library's error bound, not bit for bit.
+ * Tiles of 64 rows are centred on their centroid or on that of a near tile.
+ * mode -1 (the default): the Gram on the tensor cores where tile pairs x
+ * (d - 6) reach 65,536 and d 12 (20 for independent sets); 1: always (sets:
+ * while its buffers stay within 16 GiB); 0: never.  Process-wide; other
+ * values -> INVALID_ARG. */
 isoclust_status isoclust_set_omega_gram(int32_t mode);
 
 /* Pruned Boruvka rounds for one-set calls (Section 3.5's minimum spanning

@@ -21,22 +21,35 @@ cudaError_t weights_launch_sym(const float *X, int64_t n, int32_t d, double sigm
                                const unsigned long long *nnbits, double *omega, void *part,
                                unsigned long long *tile_counts, const uint8_t *need, cudaEvent_t *kev,
                                cudaStream_t s, const Shard *sh = nullptr, double *part64 = nullptr,
-                               OmegaGram *og = nullptr, uint32_t *status = nullptr, uint64_t wait_cycles = 0);
+                               void *gram = nullptr, uint32_t *status = nullptr, uint64_t wait_cycles = 0);
 float omega_zskip(int64_t n);
 size_t weights64_bytes(int64_t n, bool with_p);
 cudaError_t weights64_launch(const void *X, int64_t n, int32_t d, int dtype, double sigma, double alpha,
                              int include_self, double *omega, double *p, void *part, cudaStream_t s);
 constexpr size_t SYM_PART_LIMIT = size_t(16) << 30;   // symmetric sweep up to 16 GiB of partials
-// the omega Gram goes to the tensor cores by default for rows at least this
-// long (measured on GB300: 1.23x faster at d = 64, 1.3x at d = 128, 5x at
-// d = 4,096 than the double-word CUDA-core sums)
-constexpr int32_t OMEGA_GRAM_MIN_D = 64;
+// omega's Gram goes to the tensor cores by default when the tile pairs times
+// the dimensions (but for a few) outweigh its set-up (digit planes, block list:
+// some 80 us) and the one block per SM.  The omega stage in ms, CUDA cores /
+// Gram, by 64 x 64 tile pairs of the upper triangle (blobs):
+//      300 pairs: d = 64 .235/.310, 96 .286/.406
+//    1,128:       d = 48 .360/.395, 64 .410/.390
+//    4,465:       d = 16 .514/.555, 24 .596/.554, 64 1.04/.68
+//   12,403:       d = 8 .843/.941, 12 .957/.940, 32 1.51/.99
+//   49,141:       d = 8 2.77/2.63, 12 3.17/2.47, 64 9.1/2.9
+// Independent sets have more half-empty blocks; 200 sets, 50,000 pairs:
+// d = 16 3.72/3.87, 24 4.05/3.48, 32 6.08/4.21; 32 sets, 250 pairs: 96 .155/.221.
+constexpr int64_t OMEGA_GRAM_MIN_WORK = 65536;        // tile pairs x (d - 6)
+constexpr int32_t OMEGA_GRAM_MIN_D = 12, OMEGA_GRAM_SETS_MIN_D = 20;
+static bool omega_gram_pays(int64_t items, int32_t d, int32_t min_d) {
+    return d >= min_d && items * (d - 6) >= OMEGA_GRAM_MIN_WORK;
+}
 size_t weights_sym_sets_bytes(int64_t n_pad, int64_t nitems, int32_t d);
 cudaError_t weights_launch_sym_sets(const float *Xp, int64_t n_pad, int32_t d, double sigma, int include_self,
                                     const unsigned long long *nnbits, double *omega, void *part, const int2 *witems,
                                     int64_t nitems, const int32_t *tile_valid, const int32_t *tile_set,
                                     const int64_t *tile0, const int64_t *ntl, const int64_t *item0, int64_t max_n,
-                                    unsigned long long *tile_counts, cudaEvent_t *kev, cudaStream_t s);
+                                    unsigned long long *tile_counts, cudaEvent_t *kev, cudaStream_t s,
+                                    void *gram = nullptr, uint32_t *status = nullptr, uint64_t wait_cycles = 0);
 
 size_t adjoint_bytes(int64_t n, int32_t d, int32_t k);
 cudaError_t adjoint_launch(const void *X, int32_t dtype, int64_t n, int32_t d, const double *scale, double sigma,
@@ -55,7 +68,7 @@ static thread_local char g_err[512] = "";
 static thread_local double g_prof_ms[6] = {0, 0, 0, 0, 0, 0};
 static thread_local int64_t g_prof_cnt[4] = {0, 0, 0, 0};
 static thread_local int64_t g_prof_mst_tiles[2] = {0, 0};     // tile pairs swept, and a full sweep's
-static thread_local unsigned long long g_prof_tiles[3] = {0, 0, 0};
+static thread_local unsigned long long g_prof_tiles[4] = {0, 0, 0, 0};
 static thread_local int g_prof_sym = 0;
 static thread_local double g_prof_omega_kernel_ms = 0.0;
 static thread_local double g_prof_omega_gram_ms = 0.0;
@@ -153,35 +166,6 @@ void *scratch_acquire(size_t bytes, cudaStream_t stream, isoclust_status *st) {
     }
     g_scratch[dev] = p;
     g_scratch_cap[dev] = want;
-    return p;
-}
-
-static void *g_gram[MAX_DEV] = {nullptr};
-static size_t g_gram_cap[MAX_DEV] = {0};
-
-// Caller holds g_call_mu[dev] (one call per device at a time).
-void *gram_acquire(size_t bytes) {
-    int dev = current_device();
-    if (g_gram_cap[dev] >= bytes && g_gram[dev]) return g_gram[dev];
-    if (g_gram[dev]) {
-        cudaDeviceSynchronize();
-        cudaFree(g_gram[dev]);
-        g_gram[dev] = nullptr;
-        g_gram_cap[dev] = 0;
-    }
-    size_t want = bytes + bytes / 8 + (1u << 20);
-    void *p = nullptr;
-    if (cudaMalloc(&p, want) != cudaSuccess) {
-        cudaGetLastError();
-        want = bytes;
-        if (cudaMalloc(&p, want) != cudaSuccess) {
-            cudaGetLastError();
-            set_error("cannot allocate %zu bytes for the omega Gram tiles", bytes);
-            return nullptr;
-        }
-    }
-    g_gram[dev] = p;
-    g_gram_cap[dev] = want;
     return p;
 }
 
@@ -380,7 +364,7 @@ static int g_last_graph_mode = 0;                  // 0 eager, 1 captured, 2 rep
 
 static std::atomic<int> g_graphs_on{1};          // isoclust_set_batched_graphs
 static std::atomic<int> g_stall_test{0};         // isoclust_set_test_stalled_wait
-static std::atomic<int> g_omega_gram{-1};        // isoclust_set_omega_gram (-1: by row length)
+static std::atomic<int> g_omega_gram{-1};        // isoclust_set_omega_gram (-1: by size)
 static bool graphs_enabled() { return g_graphs_on.load(std::memory_order_relaxed) != 0; }
 
 struct Fnv {
@@ -409,6 +393,12 @@ static isoclust_status use_tc_sweep(const isoclust_opts &o, int dtype, bool *out
         *out = tc_supported();
     }
     return ISOCLUST_OK;
+}
+
+// 64-row tile pairs of one set's upper triangle
+static int64_t tri_items(int64_t n) {
+    const int64_t T = ceil_div(n, 64);
+    return T * (T + 1) / 2;
 }
 
 // ---------------------------------------------------------------- the pipeline
@@ -478,10 +468,9 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     const bool symmetric = permuted && o.alpha == 0.0 && o.omega_mode == ISOCLUST_OMEGA_FULL &&
                            weights_sym_bytes(n, d) <= SYM_PART_LIMIT;
     // eq. omega's Gram on the tensor cores (with the tensor-core screen)
-    int64_t gram_blocks = 0;
     const int gram_mode = g_omega_gram.load(std::memory_order_relaxed);
-    const bool gram = symmetric && use_tc && ceil_div(n, 128) <= 65535 &&
-                      (gram_mode == 1 || (gram_mode < 0 && d >= OMEGA_GRAM_MIN_D));
+    const bool gram = symmetric && use_tc &&
+                      (gram_mode == 1 || (gram_mode < 0 && omega_gram_pays(tri_items(n), d, OMEGA_GRAM_MIN_D)));
     const bool weights64 = need_labels && dtype == ISOCLUST_F64 &&
                            (o.omega_mode == ISOCLUST_OMEGA_FULL || o.alpha != 0.0) &&
                            weights64_bytes(n, o.alpha != 0.0) <= SYM_PART_LIMIT;
@@ -505,13 +494,13 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
             P.kbuf = A.take<uint64_t>(n);
             P.Xp = A.take<float>((size_t)n * d);
             P.nnp = A.take<unsigned long long>(n);
-            P.tiles = A.take<unsigned long long>(3);
+            P.tiles = A.take<unsigned long long>(4);
             P.omp = A.take<double>(n);
             P.pp = A.take<double>(n);
             if (symmetric) P.sym = (void *)A.take<unsigned char>(weights_sym_bytes(n, d));
             if (symmetric && use_tc) P.need = A.take<uint8_t>((size_t)ceil_div(n, 64) * ceil_div(n, 64));
             if (sh) P.part64 = A.take<double>(n);
-            if (gram) P.gram = (void *)A.take<unsigned char>(omega_gram_bytes(n, d), 1024);
+            if (gram) P.gram = (void *)A.take<unsigned char>(omega_tc_bytes(n, d, tri_items(n)), 1024);
         }
     };
     MstScratch M;
@@ -591,7 +580,7 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
                 ISO_CUDA(sort_pairs_u64(P.key, P.perm, P.kbuf, P.vbuf, n, s));
                 k_gather_rows<<<(unsigned)ceil_div(n * (int64_t)d, TPB), TPB, 0, ISO_S(s)>>>(
                     (const float *)X, P.perm, M.nnbits, n, d, P.Xp, P.nnp);
-                ISO_CUDA(cudaMemsetAsync(P.tiles, 0, 3 * sizeof(unsigned long long), s));
+                ISO_CUDA(cudaMemsetAsync(P.tiles, 0, 4 * sizeof(unsigned long long), s));
                 if (symmetric) {
                     // the tensor cores decide which pairs of 64-row tiles can hold a term
                     if (use_tc) {
@@ -599,13 +588,9 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
                                                  ceil_div(n, 64), s));
                         k_or_err_api<<<1, 1, 0, ISO_S(s)>>>(TC.err, status);
                     }
-                    OmegaGram og;
-                    og.scratch = P.gram;
-                    og.scratch_bytes = gram ? omega_gram_bytes(n, d) : 0;
                     ISO_CUDA(weights_launch_sym(P.Xp, n, d, sigma, o.include_self, P.nnp, P.omp, P.sym, P.tiles,
                                                 use_tc ? P.need : nullptr, ev.ok ? ev.e + 8 : nullptr, s, sh,
-                                                P.part64, gram ? &og : nullptr, status, o.spin_limit));
-                    gram_blocks = og.nblocks;
+                                                P.part64, gram ? P.gram : nullptr, status, o.spin_limit));
                 }
                 else
                     ISO_CUDA(weights_launch(P.Xp, n, d, dtype, false, sigma, o.alpha, o.include_self, P.nnp, P.omp,
@@ -668,13 +653,12 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
         g_prof_mst_tiles[0] = g_prof_mst_tiles[1];
         if (mst_pruned) g_prof_mst_tiles[0] = (int64_t)mst_swept;     // every round pruned
     }
-    g_prof_tiles[0] = g_prof_tiles[1] = g_prof_tiles[2] = 0;
+    memset(g_prof_tiles, 0, sizeof(g_prof_tiles));
     if (permuted) ISO_CUDA(cudaMemcpy(g_prof_tiles, P.tiles, sizeof(g_prof_tiles), cudaMemcpyDeviceToHost));
     g_prof_sym = symmetric ? (gram ? 3 : (use_tc ? 2 : 1)) : 0;
-    // the symmetric sweep kernel (after the Gram kernel when that ran), and the Gram kernel
-    g_prof_omega_kernel_ms = symmetric ? (gram ? ev.ms(11, 9) : ev.ms(8, 9)) : 0.0;
-    g_prof_omega_gram_ms = (symmetric && gram) ? ev.ms(10, 11) : 0.0;
-    g_prof_omega_gram_blocks = (symmetric && gram) ? gram_blocks : 0;
+    g_prof_omega_kernel_ms = symmetric ? ev.ms(8, 9) : 0.0;
+    g_prof_omega_gram_ms = (symmetric && gram) ? g_prof_omega_kernel_ms : 0.0;
+    g_prof_omega_gram_blocks = (symmetric && gram) ? (int64_t)g_prof_tiles[3] : 0;
     return map_status(fin, false);
 }
 
@@ -853,8 +837,12 @@ static isoclust_status cluster_sets_impl(const void *X, const int64_t *offsets, 
         int64_t *pos;
         float *Xp;
         unsigned long long *nnp, *tiles;
-        void *sym;
+        void *sym, *gram = nullptr;
     } B;
+    const int gram_mode = g_omega_gram.load(std::memory_order_relaxed);
+    // (many sets: within the same limit as the partials of one)
+    const bool gram = nitems > 0 && omega_tc_bytes(n_pad64, d, nitems) <= SYM_PART_LIMIT &&
+                      (gram_mode == 1 || (gram_mode < 0 && omega_gram_pays(nitems, d, OMEGA_GRAM_SETS_MIN_D)));
     auto carve = [&](Arena &A) {
         B.status = A.take<uint32_t>(4);
         B.plan = A.take<int64_t>(plan.size());
@@ -878,7 +866,8 @@ static isoclust_status cluster_sets_impl(const void *X, const int64_t *offsets, 
         B.Xp = A.take<float>((size_t)n_pad64 * d);
         B.nnp = A.take<unsigned long long>(n_pad64);
         B.omp = A.take<double>(n_pad64);
-        B.tiles = A.take<unsigned long long>(3);
+        B.tiles = A.take<unsigned long long>(4);
+        if (gram) B.gram = (void *)A.take<unsigned char>(omega_tc_bytes(n_pad64, d, nitems), 1024);
         B.sym = (void *)A.take<unsigned char>(weights_sym_sets_bytes(n_pad64, nitems, d));
     };
     Arena meas;
@@ -956,10 +945,10 @@ static isoclust_status cluster_sets_impl(const void *X, const int64_t *offsets, 
         if ((e = cudaMemsetAsync(B.nnp, 0xff, sizeof(unsigned long long) * n_pad64, q))) return e;
         k_gather_pad<<<(unsigned)ceil_div(N * (int64_t)d, TPB), TPB, 0, ISO_S(q)>>>((const float *)X, B.pos, M.nnbits, N,
                                                                                     d, B.Xp, B.nnp);
-        if ((e = cudaMemsetAsync(B.tiles, 0, 3 * sizeof(unsigned long long), q))) return e;
+        if ((e = cudaMemsetAsync(B.tiles, 0, 4 * sizeof(unsigned long long), q))) return e;
         if ((e = weights_launch_sym_sets(B.Xp, n_pad64, d, sigma, o.include_self, B.nnp, B.omp, B.sym, B.witems,
                                          nitems, B.tile_valid, B.tile_set, d_tile0, d_ntl, d_item0, max_n, B.tiles,
-                                         E.ok ? E.e + 8 : nullptr, q)))
+                                         E.ok ? E.e + 8 : nullptr, q, B.gram, B.status, o.spin_limit)))
             return e;
         k_scatter_pad<<<(unsigned)ceil_div(N + 1, TPB), TPB, 0, ISO_S(q)>>>(B.omp, B.pos, N, B.om);
         E.rec(4, q);
@@ -1061,10 +1050,10 @@ static isoclust_status cluster_sets_impl(const void *X, const int64_t *offsets, 
     g_prof_cnt[2] = DP_TREE_PASSES + 1;
     g_prof_cnt[3] = 0;
     ISO_CUDA(cudaMemcpy(g_prof_tiles, B.tiles, sizeof(g_prof_tiles), cudaMemcpyDeviceToHost));
-    g_prof_sym = 1;
+    g_prof_sym = gram ? 3 : 1;
     g_prof_omega_kernel_ms = nitems > 0 ? E.ms(8, 9) : 0.0;
-    g_prof_omega_gram_ms = 0.0;
-    g_prof_omega_gram_blocks = 0;
+    g_prof_omega_gram_ms = gram ? g_prof_omega_kernel_ms : 0.0;
+    g_prof_omega_gram_blocks = gram ? (int64_t)g_prof_tiles[3] : 0;
     return map_status(fin, false);
 }
 

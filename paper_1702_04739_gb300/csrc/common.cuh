@@ -91,31 +91,27 @@ struct Arena {
 // Per-device cached scratch (grow-only).  Returns nullptr on failure.
 void *scratch_acquire(size_t bytes, cudaStream_t stream, isoclust_status *st);
 void scratch_release();
-// A second per-device cached buffer (grow-only) for the omega Gram tiles,
-// whose size is known only after the screen.  nullptr on failure.
-void *gram_acquire(size_t bytes);
 
-// The Gram of eq. omega's tile pairs on the tensor cores (omega_tc.cu).
-// scratch / scratch_bytes: omega_gram_bytes(n, d) bytes of the call's
-// scratch; the launch fills the rest (rows of the omega order padded to 128).
-struct OmegaGram {
-    void *scratch = nullptr;
-    size_t scratch_bytes = 0;
-    float *yh = nullptr, *yl = nullptr;   // [n_pad][d] y = x - c_T as a double-word
-    int32_t *rexp = nullptr;              // [n_pad] E of each row
-    float2 *rnorm = nullptr;              // [n_pad] |y|^2 as a double-word
-    int32_t *item_slot = nullptr;         // [items] 2 x block + half, -1 when the screen drops the item
-    float2 *gbuf = nullptr;               // [blocks][128][64] G in units of 2^(E_i + E_j - 14)
-    int64_t nblocks = 0;
-    int one_centre = 0;                   // every row centred on one point instead of its tile's centroid
+// The 64-row tile pairs of an omega sweep (omega_tc.cu, weights.cu): one set's
+// upper triangle (T tiles of n rows), or a list for independent sets (witems,
+// with each tile's set, real rows and the sets' tile and item offsets).
+struct OmegaItems {
+    int64_t nitems = 0, T = 0, n = 0;
+    const int2 *witems = nullptr;
+    const int32_t *tile_set = nullptr, *tile_valid = nullptr;
+    const int64_t *tile0 = nullptr, *ntl = nullptr, *item0 = nullptr;
 };
-// Rows at least this long are centred on one point for the Gram (no cross terms).
-constexpr int32_t OMEGA_ONE_CENTRE_MIN_D = 1024;
-size_t omega_gram_bytes(int64_t n, int32_t d);
-// kev (may be null): two events recorded around the Gram kernel
-cudaError_t omega_gram_launch(OmegaGram &G, const float *Xp, int64_t n, int32_t d, const float *cen,
-                              const uint8_t *tskip, uint32_t *err, uint64_t wait_cycles, cudaStream_t s,
-                              cudaEvent_t *kev = nullptr);
+struct ExpTable;
+// Scratch of omega_tc_launch for `rows` rows of the omega order.
+size_t omega_tc_bytes(int64_t rows, int32_t d, int64_t nitems);
+// The kept tile pairs' terms (tskip 0) with the Gram on the tensor cores:
+// row and column partials and flags as k_weights_sym writes them.
+// kev (may be null): two events recorded around the kernel.
+cudaError_t omega_tc_launch(void *scratch, size_t scratch_bytes, const OmegaItems &L, const float *Xp, int64_t rows,
+                            int32_t d, const float *cen, const float2 *shdw, const uint8_t *tskip, float is_h, float is_l,
+                            float zskip, const ExpTable &tab, uint8_t *flags, float2 *rpart, float2 *cpart,
+                            unsigned long long *tile_counts, int shard_rank, int shard_world, uint32_t *err,
+                            uint64_t wait_cycles, cudaStream_t s, cudaEvent_t *kev);
 
 // ---------------------------------------------------------------- helpers
 __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }

@@ -61,10 +61,10 @@ __device__ __forceinline__ void dw_exp_neg(float zh, float zl, const float2 *__r
     const float poly = __fmaf_rn(__fmaf_rn(-1.0f / 120.0f, rh, 1.0f / 24.0f), rh, -1.0f / 6.0f);
     const float tail = __fmul_rn(__fmul_rn(s2, rh), poly);
     float eh, el;
-    two_sum(1.0f, -rh, eh, el);
+    fast_two_sum(1.0f, -rh, eh, el);               // 1 > |rh|: exact
     el = __fadd_rn(__fsub_rn(el, rl), __fadd_rn(h2e, tail));
     float eh2, el2;
-    two_sum(eh, h2, eh2, el2);
+    fast_two_sum(eh, h2, eh2, el2);                // eh > h2: exact
     el2 = __fadd_rn(el2, el);
     float mh, ml;
     fast_two_sum(eh2, el2, mh, ml);

@@ -8,10 +8,11 @@
 #include "common.cuh"
 
 namespace iso {
-// TMA map of a row-major BF16 array (rows x cols, cols a multiple of 64, the
-// row pitch cols * 2 bytes): boxes of 64 columns (128 bytes, 128-byte
-// swizzle) by box_rows rows.  Host function (mst_tc.cu).
-cudaError_t tc_map_bf16(CUtensorMap *m, const void *base, int64_t rows, int32_t cols, int box_rows);
+// TMA map of a row-major BF16 array (rows x cols, cols a multiple of box_cols,
+// the row pitch cols * 2 bytes): boxes of box_cols columns (64: 128 bytes with
+// the 128-byte swizzle; 32: 64 bytes with the 64-byte swizzle) by box_rows
+// rows.  Host function (mst_tc.cu).
+cudaError_t tc_map_bf16(CUtensorMap *m, const void *base, int64_t rows, int32_t cols, int box_rows, int box_cols = 64);
 
 namespace tcx {
 
@@ -87,6 +88,18 @@ __device__ __forceinline__ uint64_t make_sw128_desc(uint32_t saddr) {
     d |= (uint64_t)(1024u >> 4) << 32;       // stride byte offset
     d |= (uint64_t)1 << 46;                  // descriptor version
     d |= (uint64_t)2 << 61;                  // 128-byte swizzle
+    return d;
+}
+
+// The same with the 64-byte swizzle: rows of 64 bytes, 8-row groups 512 bytes
+// apart.
+__device__ __forceinline__ uint64_t make_sw64_desc(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(512u >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;                  // 64-byte swizzle
     return d;
 }
 

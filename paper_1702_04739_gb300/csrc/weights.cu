@@ -43,8 +43,6 @@ constexpr int TPB = 256;
 constexpr int WT = 64;        // rows / columns per tile
 constexpr int WDC = 32;       // dims per shared-memory chunk
 constexpr int WPAD = WT + 4;
-constexpr int GR_DCH = (WDC * WPAD) / 2;    // dimensions of D per chunk (a double-word each, in As)
-constexpr int GR_FCAP = (WDC * WPAD) / 2;   // cancelling pairs per round (indices in Bs, results in As)
 
 struct RowAcc {
     float wh, wl, ph, pl;
@@ -376,28 +374,6 @@ __global__ void k_tile_pair_skip(const float *__restrict__ cen, const float *__r
     }
 }
 
-// d2 of rows of the omega order from the tensor-core Gram (omega_tc.cu).
-struct GramArgs {
-    const float2 *gbuf;          // [blocks][128][64] G in units of 2^(E_i + E_j - 14)
-    const int32_t *item_slot;    // per item: 2 x block + half
-    const float *yh, *yl;        // y = x - c_T, double-word
-    const int32_t *rexp;         // E of each row
-    const float2 *rnorm;         // |y|^2, double-word
-    const float *cen;            // tile centroids c_T
-    int one_centre;              // 1: every row was centred on the same point (D = 0)
-};
-
-// 16-byte asynchronous global -> shared copies (the Gram tile of an item,
-// landing while the item's cross terms are computed)
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
-                 "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-constexpr int GR_GTILE_BYTES = WT * WT * (int)sizeof(float2);      // one item's Gram tile (32 KB)
-
 // Symmetric omega sweep: each unordered tile pair is screened in FP32 and,
 // if any of its terms can matter in either direction, evaluated once in
 // double-word arithmetic; the pair's d2 serves both omega_i and omega_j.
@@ -405,14 +381,14 @@ constexpr int GR_GTILE_BYTES = WT * WT * (int)sizeof(float2);      // one item's
 // of item w, so the final sums do not depend on scheduling.
 // Independent sets: the tile pairs come from a list (both tiles of one set)
 // and tile_valid[I] counts the real rows of tile I (padding follows them).
-template <bool SETS, bool GRAM = false>
+template <bool SETS>
 __global__ void __launch_bounds__(TPB, 2)
 k_weights_sym(const float *__restrict__ X, int64_t n, int32_t d, const float2 *__restrict__ shdw,
               float is_h, float is_l, ExpTable tabv, float zskip, float scr_shrink, int64_t T,
               int64_t nitems, const int2 *__restrict__ witems, const int32_t *__restrict__ tile_valid,
               const uint8_t *__restrict__ tskip, int prescreened, uint8_t *__restrict__ flags,
               float2 *__restrict__ rpart, float2 *__restrict__ cpart, unsigned long long *__restrict__ tile_counts,
-              int shard_rank, int shard_world, GramArgs ga) {
+              int shard_rank, int shard_world) {
     __shared__ __align__(16) float As[WDC][WPAD];
     __shared__ __align__(16) float Bs[WDC][WPAD];
     __shared__ float2 tab[64];
@@ -420,16 +396,10 @@ k_weights_sym(const float *__restrict__ X, int64_t n, int32_t d, const float2 *_
     __shared__ float2 mc[WT][17];
     __shared__ int64_t sIJ[5];
     __shared__ float sred[TPB / 32][2];        // per warp: smallest and largest shift of its real rows
-    __shared__ float2 sUV[GRAM ? 2 * WT : 1];  // GRAM: |y|^2 +- 2 <y, D> of the rows of I, then of J
-    __shared__ float sSc[GRAM ? 2 * WT : 1];   // GRAM: 2^(E - 7) of the rows of I, 2^(E - 6) of J
-    __shared__ float2 sC;                      // GRAM: |D|^2
-    __shared__ float sMg[GRAM ? 2 * WT : 1];   // GRAM: |y|^2 + 2 |<y, D>| (+ |D|^2 for I): the parts' size
-    __shared__ int sFb;                        // GRAM: cancelling pairs of the item
-    extern __shared__ __align__(16) float2 sG[];   // GRAM: the item's Gram tile, [WT][WT] double-words
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
     if (tid < 64) tab[tid] = tabv.t[tid];
-    unsigned long long dw_items = 0, screened = 0, fallbacks = 0;
+    unsigned long long dw_items = 0, screened = 0;
     // a sharded call evaluates the items w with w mod world == rank
     for (int64_t w = (int64_t)blockIdx.x * shard_world + shard_rank; w < nitems;
          w += (int64_t)gridDim.x * shard_world) {
@@ -536,243 +506,12 @@ k_weights_sym(const float *__restrict__ X, int64_t n, int32_t d, const float2 *_
             }
         }
         ++dw_items;
-        if constexpr (GRAM) {
-            // the item's Gram tile into shared memory (it lands during the
-            // cross terms; every reader of the previous tile is past the
-            // item's first barrier)
-            const int32_t gslot = ga.item_slot[w];
-            if (gslot >= 0) {
-                const float4 *src = reinterpret_cast<const float4 *>(
-                    ga.gbuf + ((size_t)(gslot >> 1) * (2 * WT) + (size_t)(gslot & 1) * WT) * WT);
-                float4 *dst = reinterpret_cast<float4 *>(sG);
-#pragma unroll
-                for (int q = 0; q < GR_GTILE_BYTES / 16 / TPB; ++q) cp_async16(dst + tid + q * TPB, src + tid + q * TPB);
-            }
-            cp_async_commit();
-        }
         // ---- double-word pass
         float S[4][4], E[4][4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int j = 0; j < 4; ++j) { S[i][j] = 0.f; E[i][j] = 0.f; }
-        if constexpr (GRAM) {
-            // d2 = (|y_i|^2 + 2 <y_i, D> + |D|^2) + (|y_j|^2 - 2 <y_j, D>) - 2 G_ij, y = x - c_T,
-            // D = c_I - c_J (zero on the diagonal and when every row shares one centre)
-            const int lane = tid & 31, wq = tid >> 5;
-            const bool cross = !diag && !ga.one_centre;
-            float2 *sD = reinterpret_cast<float2 *>(&As[0][0]);          // D chunk, double-word
-            float2 *sX = reinterpret_cast<float2 *>(&Bs[0][0]);          // upper half's partial products
-            {
-                // products p = 0..63 (rows of I) and 64..127 (rows of J), one
-                // thread each; the two halves of the block take alternate
-                // dimensions of every chunk of D
-                const int pr = tid & 127, hh = tid >> 7;
-                const int64_t gr = pr < WT ? row0 + pr : col0 + (pr - WT);
-                float xh = 0.f, xl = 0.f, ch = 0.f, cl = 0.f;
-                if (cross) {
-                    const float *cI = ga.cen + I * d, *cJ = ga.cen + J * d;
-                    const float *ryh = ga.yh + gr * d, *ryl = ga.yl + gr * d;
-                    for (int t0 = 0; t0 < d; t0 += GR_DCH) {
-                        const int tl = min(GR_DCH, d - t0);
-                        __syncthreads();                       // previous chunk's readers are done
-                        for (int t = tid; t < tl; t += TPB) {
-                            float Dh, Dl;
-                            two_sum(cI[t0 + t], -cJ[t0 + t], Dh, Dl);
-                            sD[t] = make_float2(Dh, Dl);
-                            float p, e;
-                            two_prod(Dh, Dh, p, e);
-                            e = __fmaf_rn(__fadd_rn(Dh, Dh), Dl, e);
-                            dw_add(ch, cl, p, e);
-                        }
-                        __syncthreads();
-                        // the lower half of the block takes the chunk's first
-                        // h4 dimensions, the upper half the rest (4 at a time
-                        // when rows are 16-byte aligned)
-                        const int h4 = ((tl + 7) >> 3) << 2;
-                        const int ta = hh ? min(h4, tl) : 0, tb = hh ? tl : min(h4, tl);
-                        auto term = [&](float a, float al, float2 D) {
-                            float p, e;
-                            two_prod(a, D.x, p, e);
-                            e = __fmaf_rn(a, D.y, __fmaf_rn(al, D.x, e));
-                            dw_add(xh, xl, p, e);
-                        };
-                        if ((d & 3) == 0) {
-                            for (int t = ta; t < tb; t += 4) {
-                                const float4 a4 = *reinterpret_cast<const float4 *>(ryh + t0 + t);
-                                const float4 l4 = *reinterpret_cast<const float4 *>(ryl + t0 + t);
-                                const float4 d01 = *reinterpret_cast<const float4 *>(sD + t);
-                                const float4 d23 = *reinterpret_cast<const float4 *>(sD + t + 2);
-                                term(a4.x, l4.x, make_float2(d01.x, d01.y));
-                                term(a4.y, l4.y, make_float2(d01.z, d01.w));
-                                term(a4.z, l4.z, make_float2(d23.x, d23.y));
-                                term(a4.w, l4.w, make_float2(d23.z, d23.w));
-                            }
-                        } else {
-                            for (int t = ta; t < tb; ++t) term(ryh[t0 + t], ryl[t0 + t], sD[t]);
-                        }
-                    }
-                    // |D|^2: the threads' chunk partials, folded in a fixed order
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const float oh = __shfl_xor_sync(0xffffffffu, ch, o);
-                        const float ol = __shfl_xor_sync(0xffffffffu, cl, o);
-                        dw_add(ch, cl, oh, ol);
-                    }
-                    if (hh) sX[pr] = make_float2(xh, xl);
-                }
-                __syncthreads();
-                if (cross && lane == 0) sX[128 + wq] = make_float2(ch, cl);
-                __syncthreads();
-                if (tid < 2 * WT) {
-                    const float2 rn = ga.rnorm[gr];
-                    float uh = rn.x, ul = rn.y;
-                    float mg = rn.x;
-                    if (cross) {
-                        const float2 o = sX[pr];
-                        dw_add(xh, xl, o.x, o.y);
-                        const float sg = pr < WT ? 2.0f : -2.0f;
-                        dw_add(uh, ul, __fmul_rn(sg, xh), __fmul_rn(sg, xl));
-                        mg = __fadd_rn(rn.x, fabsf(__fmul_rn(2.0f, xh)));
-                    }
-                    sUV[pr] = make_float2(uh, ul);
-                    sMg[pr] = mg;
-                    sSc[pr] = ldexpf(1.0f, ga.rexp[gr] - (pr < WT ? 7 : 6));
-                }
-                if (tid == 0) {
-                    float h = 0.f, l = 0.f;
-                    if (cross)
-                        for (int q = 0; q < TPB / 32; ++q) dw_add(h, l, sX[128 + q].x, sX[128 + q].y);
-                    sC = make_float2(h, l);
-                }
-            }
-            cp_async_wait_all();
-            __syncthreads();
-            const int32_t slot = ga.item_slot[w];
-            // (every kept item has a Gram block; should one lack it, its pairs
-            // take the direct sums below)
-            const float2 *Gp = sG;
-            const float2 C = sC;
-            unsigned fb = 0u;                  // pairs whose Gram form cancels (bit 4i + j)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int lr = ty * 4 + i;
-                float uh = sUV[lr].x, ul = sUV[lr].y;
-                dw_add(uh, ul, C.x, C.y);
-                const float mi = sMg[lr] + C.x, si = sSc[lr];
-                float4 g01 = make_float4(0.f, 0.f, 0.f, 0.f), g23 = g01;
-                if (slot >= 0) {
-                    g01 = *reinterpret_cast<const float4 *>(Gp + lr * WT + tx * 4);
-                    g23 = *reinterpret_cast<const float4 *>(Gp + lr * WT + tx * 4 + 2);
-                }
-                const float gv[4][2] = {{g01.x, g01.y}, {g01.z, g01.w}, {g23.x, g23.y}, {g23.z, g23.w}};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int lc = tx * 4 + j;
-                    const float sc = __fmul_rn(si, sSc[WT + lc]);      // 2^(E_i + E_j - 13), exact
-                    const float gh = __fmul_rn(gv[j][0], sc), gl = __fmul_rn(gv[j][1], sc);
-                    const float2 V = sUV[WT + lc];
-                    float h = uh, l = ul;
-                    dw_add(h, l, V.x, V.y);
-                    dw_add(h, l, -gh, -gl);
-                    // the Gram form's error is about 2^-46 of the addends'
-                    // size M: where they cancel to under half of it, the
-                    // pair takes the direct sum of squared differences
-                    const float M = mi + sMg[WT + lc] + fabsf(gh);
-                    const bool real = rok(lr) && cok(lc) && !(diag && lc == lr);
-                    if (real && (slot < 0 || !(__fmul_rn(h, 2.0f) >= M))) fb |= 1u << (4 * i + j);
-                    S[i][j] = h;
-                    E[i][j] = l;
-                }
-            }
-            fallbacks += (unsigned)__popc(fb);
-            // the cancelling pairs go to a block-wide list (pair index lr * 64
-            // + lc), evaluated by groups of GL lanes (a lane per GL-th
-            // dimension, the group's double-word partials folded in a fixed
-            // tree); results come back through shared memory
-            uint16_t *flist = reinterpret_cast<uint16_t *>(&Bs[0][0]);
-            float2 *fres = reinterpret_cast<float2 *>(&As[0][0]);
-            if (tid == 0) sFb = 0;
-            __syncthreads();
-            const int nmine = __popc(fb);
-            const int fbase = nmine ? atomicAdd(&sFb, nmine) : 0;
-            __syncthreads();
-            const int ftotal = sFb;
-            const int GL = d >= 256 ? 32 : 8;
-            const int ngroups = (TPB / 32) * (32 / GL);      // groups in the block
-            for (int r0 = 0; r0 < ftotal; r0 += GR_FCAP) {
-                const int rn = min(GR_FCAP, ftotal - r0);
-                {
-                    unsigned m = fb;
-                    for (int q = 0; m; ++q) {
-                        const int b = __ffs(m) - 1;
-                        m &= m - 1u;
-                        const int e = fbase + q - r0;
-                        if (e >= 0 && e < rn) flist[e] = (uint16_t)((ty * 4 + (b >> 2)) * WT + tx * 4 + (b & 3));
-                    }
-                }
-                __syncthreads();
-                {
-                    // warp-uniform trip count: the groups of a warp take
-                    // consecutive entries, the whole warp shuffles
-                    const int gpw = 32 / GL, wg = lane / GL, gl = lane % GL;
-                    for (int eb = wq * gpw; eb < rn; eb += ngroups) {
-                        const int e = eb + wg;
-                        float ph = 0.f, pl = 0.f;
-                        if (e < rn) {
-                            const int pi = flist[e];
-                            const float *xa = X + (row0 + (pi >> 6)) * d, *xb = X + (col0 + (pi & 63)) * d;
-                            auto sq = [&](float a, float b) {
-                                float s1, e1;
-                                two_sum(a, -b, s1, e1);
-                                const float p = __fmul_rn(s1, s1);
-                                float q2 = __fmaf_rn(s1, s1, -p);
-                                q2 = __fmaf_rn(__fadd_rn(s1, s1), e1, q2);
-                                dw_add(ph, pl, p, q2);
-                            };
-                            if ((d & 3) == 0) {
-                                // 4 consecutive dimensions per lane and step
-                                for (int t = 4 * gl; t < d; t += 4 * GL) {
-                                    const float4 a = *reinterpret_cast<const float4 *>(xa + t);
-                                    const float4 b = *reinterpret_cast<const float4 *>(xb + t);
-                                    sq(a.x, b.x);
-                                    sq(a.y, b.y);
-                                    sq(a.z, b.z);
-                                    sq(a.w, b.w);
-                                }
-                            } else {
-                                for (int t = gl; t < d; t += GL) sq(xa[t], xb[t]);
-                            }
-                        }
-                        for (int o = GL >> 1; o > 0; o >>= 1) {
-                            const float oh = __shfl_xor_sync(0xffffffffu, ph, o);
-                            const float ol = __shfl_xor_sync(0xffffffffu, pl, o);
-                            dw_add(ph, pl, oh, ol);
-                        }
-                        if (e < rn && gl == 0) fres[e] = make_float2(ph, pl);
-                    }
-                }
-                __syncthreads();
-                {
-                    unsigned m = fb;
-                    for (int q = 0; m; ++q) {
-                        const int b = __ffs(m) - 1;
-                        m &= m - 1u;
-                        const int e = fbase + q - r0;
-                        if (e >= 0 && e < rn) {
-                            const float2 v = fres[e];
-#pragma unroll
-                            for (int kk = 0; kk < 16; ++kk)
-                                if (kk == b) {
-                                    S[kk >> 2][kk & 3] = v.x;
-                                    E[kk >> 2][kk & 3] = v.y;
-                                }
-                        }
-                    }
-                }
-                __syncthreads();
-            }
-        } else
         for (int t0 = 0; t0 < d; t0 += WDC) {
             __syncthreads();
 #pragma unroll
@@ -957,12 +696,6 @@ k_weights_sym(const float *__restrict__ X, int64_t n, int32_t d, const float2 *_
         atomicAdd(tile_counts + 0, screened);
         atomicAdd(tile_counts + 1, dw_items);
     }
-    if constexpr (GRAM) {
-        // pairs that took the direct sums (tile_counts[2])
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) fallbacks += __shfl_xor_sync(0xffffffffu, fallbacks, o);
-        if ((tid & 31) == 0 && fallbacks) atomicAdd(tile_counts + 2, fallbacks);
-    }
 }
 
 // Per row: the shift y_nn = |x - x_nn| / sigma as a double-word (once per call).
@@ -1142,11 +875,12 @@ size_t weights_sym_bytes(int64_t n, int32_t d) {
 }
 
 // Symmetric screened omega (F32 input, p not needed).  part must hold
-// weights_sym_bytes(n) bytes.
+// weights_sym_bytes(n) bytes.  gram != null: the kept tile pairs' Gram on the
+// tensor cores (omega_tc_bytes bytes; needs the tensor-core screen, need).
 cudaError_t weights_launch_sym(const float *X, int64_t n, int32_t d, double sigma, int include_self,
                                const unsigned long long *nnbits, double *omega, void *part,
                                unsigned long long *tile_counts, const uint8_t *need, cudaEvent_t *kev,
-                               cudaStream_t s, const Shard *sh, double *part64, OmegaGram *og, uint32_t *status,
+                               cudaStream_t s, const Shard *sh, double *part64, void *gram, uint32_t *status,
                                uint64_t wait_cycles) {
     static const ExpTable tab = make_exp_table();
     const double is = 1.0 / sigma;
@@ -1166,30 +900,22 @@ cudaError_t weights_launch_sym(const float *X, int64_t n, int32_t d, double sigm
     cudaError_t err;
     // sharded: the items of other ranks hold nothing here
     if (sh && (err = cudaMemsetAsync(P.flags, 0, (size_t)items, s))) return err;
-    if (kev) record_event(kev[0], s);
-    if (og && need) {
-        // the kept tile pairs' Gram on the tensor cores, then the terms
-        if ((err = omega_gram_launch(*og, X, n, d, P.cen, P.tskip, status, wait_cycles, s, kev ? kev + 2 : nullptr)))
+    if (gram && need) {
+        OmegaItems L;
+        L.nitems = items;
+        L.T = T;
+        L.n = n;
+        if ((err = omega_tc_launch(gram, omega_tc_bytes(n, d, items), L, X, n, d, P.cen, P.shdw, P.tskip, is_h, is_l, zskip,
+                                   tab, P.flags, P.rpart, P.cpart, tile_counts, sh ? sh->rank : 0, sh ? sh->world : 1,
+                                   status, wait_cycles, s, kev)))
             return err;
-        const GramArgs ga{og->gbuf, og->item_slot, og->yh, og->yl, og->rexp, og->rnorm, P.cen, og->one_centre};
-        static bool gattr = false;
-        if (!gattr) {
-            if ((err = cudaFuncSetAttribute(k_weights_sym<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            GR_GTILE_BYTES)))
-                return err;
-            gattr = true;
-        }
-        k_weights_sym<false, true><<<grid, TPB, GR_GTILE_BYTES, ISO_S(s)>>>(X, n, d, P.shdw, is_h, is_l, tab, zskip, shrink, T,
-                                                               items, nullptr, nullptr, P.tskip, 1, P.flags, P.rpart,
-                                                               P.cpart, tile_counts, sh ? sh->rank : 0,
-                                                               sh ? sh->world : 1, ga);
     } else {
+        if (kev) record_event(kev[0], s);
         k_weights_sym<false><<<grid, TPB, 0, ISO_S(s)>>>(X, n, d, P.shdw, is_h, is_l, tab, zskip, shrink, T, items,
                                                          nullptr, nullptr, P.tskip, need ? 1 : 0, P.flags, P.rpart,
-                                                         P.cpart, tile_counts, sh ? sh->rank : 0, sh ? sh->world : 1,
-                                                         GramArgs{});
+                                                         P.cpart, tile_counts, sh ? sh->rank : 0, sh ? sh->world : 1);
+        if (kev) record_event(kev[1], s);
     }
-    if (kev) record_event(kev[1], s);
     k_weights_reduce<<<(unsigned)ceil_div(n, 256), 256, 0, ISO_S(s)>>>(nnbits, n, T, is, include_self, P.flags,
                                                                       P.rpart, P.cpart, omega, sh ? part64 : nullptr);
     if (sh) {
@@ -1211,7 +937,8 @@ cudaError_t weights_launch_sym_sets(const float *Xp, int64_t n_pad, int32_t d, d
                                     const unsigned long long *nnbits, double *omega, void *part, const int2 *witems,
                                     int64_t nitems, const int32_t *tile_valid, const int32_t *tile_set,
                                     const int64_t *tile0, const int64_t *ntl, const int64_t *item0, int64_t max_n,
-                                    unsigned long long *tile_counts, cudaEvent_t *kev, cudaStream_t s) {
+                                    unsigned long long *tile_counts, cudaEvent_t *kev, cudaStream_t s, void *gram,
+                                    uint32_t *status, uint64_t wait_cycles) {
     static const ExpTable tab = make_exp_table();
     const double is = 1.0 / sigma;
     const float is_h = (float)is;
@@ -1227,15 +954,31 @@ cudaError_t weights_launch_sym_sets(const float *Xp, int64_t n_pad, int32_t d, d
     if (nitems > 0) {
         k_tile_pair_skip<true><<<(unsigned)(num_sms() * 8), 256, 0, ISO_S(s)>>>(
             P.cen, P.rad, P.msh, d, T, nitems, witems, is_h, zskip, shrink, nullptr, P.tskip);
-        if (kev) record_event(kev[0], s);
         // independent sets: the tile bound is the only screen; tile pairs it
-        // keeps go straight to the double-word pass (for sets of a few
-        // thousand points nearly every pair of tiles holds terms, so the FP32
-        // pair screen would cost more than the double-word work it saves)
-        k_weights_sym<true><<<grid, TPB, 0, ISO_S(s)>>>(Xp, n_pad, d, P.shdw, is_h, is_l, tab, zskip, shrink, 0, nitems,
-                                                        witems, tile_valid, P.tskip, 1, P.flags, P.rpart, P.cpart,
-                                                        tile_counts, 0, 1, GramArgs{});
-        if (kev) record_event(kev[1], s);
+        // keeps go straight to the pair terms (for sets of a few thousand
+        // points nearly every pair of tiles holds terms, so the FP32 pair
+        // screen would cost more than the work it saves)
+        if (gram) {
+            OmegaItems L;
+            L.nitems = nitems;
+            L.n = n_pad;
+            L.witems = witems;
+            L.tile_set = tile_set;
+            L.tile_valid = tile_valid;
+            L.tile0 = tile0;
+            L.ntl = ntl;
+            L.item0 = item0;
+            cudaError_t err = omega_tc_launch(gram, omega_tc_bytes(n_pad, d, nitems), L, Xp, n_pad, d, P.cen, P.shdw,
+                                              P.tskip, is_h, is_l, zskip, tab, P.flags, P.rpart, P.cpart, tile_counts, 0,
+                                              1, status, wait_cycles, s, kev);
+            if (err) return err;
+        } else {
+            if (kev) record_event(kev[0], s);
+            k_weights_sym<true><<<grid, TPB, 0, ISO_S(s)>>>(Xp, n_pad, d, P.shdw, is_h, is_l, tab, zskip, shrink, 0,
+                                                            nitems, witems, tile_valid, P.tskip, 1, P.flags, P.rpart,
+                                                            P.cpart, tile_counts, 0, 1);
+            if (kev) record_event(kev[1], s);
+        }
     }
     k_weights_reduce_sets<<<(unsigned)ceil_div(n_pad, 256), 256, 0, ISO_S(s)>>>(
         nnbits, n_pad, tile_valid, tile_set, tile0, ntl, item0, is, include_self, P.flags, P.rpart, P.cpart, omega);

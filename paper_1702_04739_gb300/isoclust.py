@@ -438,7 +438,7 @@ def set_batched_graphs(enable: bool) -> None:
 
 def set_omega_gram(mode) -> None:
     """eq. omega's Gram on the tensor cores: True / 1 always, False / 0 never
-    (double-word sums of squared differences), -1 by row length, the
+    (double-word sums of squared differences), -1 by size, the
     default (isoclust_set_omega_gram)."""
     _check(load().isoclust_set_omega_gram(int(mode)))
 
