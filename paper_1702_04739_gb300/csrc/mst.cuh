@@ -61,6 +61,7 @@ struct TcScratch {
     float *tv = nullptr, *tu = nullptr;            // per (list, row): best-8 candidate-block lower bounds, best upper bound
     int32_t *tj = nullptr;
     int32_t *nsurv = nullptr, *surv = nullptr;     // per row: columns to key in FP64 (padded column indices)
+    unsigned int *rmin = nullptr;                  // per row: FP32 minimum of a rescan (bits)
     uint32_t *err = nullptr;
     uint32_t *qctr = nullptr;                      // the sweep's work-item counter (zeroed before each launch)
     // independent sets (null for one set): sweep work items {row tile,

@@ -823,8 +823,12 @@ __device__ __forceinline__ void recheck_row(int64_t r, int lane, const float *__
                                             const int32_t *__restrict__ set_of, const int32_t *__restrict__ setcnt,
                                             int32_t *counters, int32_t *__restrict__ bj_s, int shard_rank,
                                             int shard_world,
-                                            const int32_t *__restrict__ row_lists, float eps64) {
-    if (lane == 0) nsurv[r] = 0;           // every row, padding included: k_exact_tc reads them all
+                                            const int32_t *__restrict__ row_lists, float eps64,
+                                            unsigned int *__restrict__ rmin) {
+    if (lane == 0) {
+        nsurv[r] = 0;                      // every row, padding included: k_exact_tc reads them all
+        rmin[r] = 0x7f800000u;
+    }
     const int64_t i = perm[r];
     if (i < 0) return;                     // padding row
     if (shard_world > 1 && (int)((r / TC_BM) % shard_world) != shard_rank) {
@@ -879,7 +883,7 @@ __device__ __forceinline__ void recheck_row(int64_t r, int lane, const float *__
     if (cnt >= TC_TOPK) {
         if (lane == 0) {
             const int q = atomicAdd(counters + MC_OVERFLOW, 1);
-            ovf[q] = (int32_t)i;
+            ovf[q] = (int32_t)r;
             rowj[i] = -2;
         }
         return;
@@ -984,7 +988,7 @@ __device__ __forceinline__ void recheck_row(int64_t r, int lane, const float *__
     if (lane == 0) {
         if (ns > TC_SURV) {                     // many near-ties: exact rescan of the row
             const int q = atomicAdd(counters + MC_OVERFLOW, 1);
-            ovf[q] = (int32_t)i;
+            ovf[q] = (int32_t)r;
             rowj[i] = -2;
         } else {
             nsurv[r] = ns;
@@ -1026,6 +1030,66 @@ __global__ void __launch_bounds__(256) k_exact_tc(const P *__restrict__ x, int b
     }
 }
 
+// The same for long rows: a warp keys one column of each of its 32 rows at a
+// time.  The squares of 32 dimensions are formed by the lanes, a dimension
+// each (whole lines of the rows), and handed over in shared memory; each lane
+// then adds its own row's in order.  (A thread per row reads a line per lane
+// and load: 1.0 ms a round at 3,279 x 1,558.)
+constexpr int EX_WIDE_MIN_D = 256;
+template <class P>
+__global__ void __launch_bounds__(128) k_exact_wide(const P *__restrict__ x, int by_point, int64_t n, int32_t d,
+                                                    const int32_t *__restrict__ perm, const int32_t *__restrict__ nsurv,
+                                                    const int32_t *__restrict__ surv, double *__restrict__ rowd2,
+                                                    int32_t *__restrict__ rowj, const int32_t *counters) {
+    if (!mst_active(counters)) return;
+    __shared__ double sq[4][32][33];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const int64_t gs = (int64_t)gridDim.x * 128;
+    for (int64_t r0 = (int64_t)blockIdx.x * 128 + wp * 32; r0 < n; r0 += gs) {
+        const int64_t r = r0 + lane;
+        const int32_t i = r < n ? perm[r] : -1;
+        int c = i >= 0 ? nsurv[r] : 0;
+        if (c > TC_SURV) c = 0;
+        double best = INFINITY;
+        int32_t bestj = -1;
+        for (int q = 0; __any_sync(0xffffffffu, q < c); ++q) {
+            int64_t jp = q < c ? surv[r * TC_SURV + q] : -1;
+            int32_t j = jp >= 0 && jp < n ? perm[jp] : -1;
+            if (j < 0) jp = -1;
+            const int64_t ra = by_point ? (int64_t)i : r, rb = by_point ? (int64_t)j : jp;
+            const unsigned live = __ballot_sync(0xffffffffu, jp >= 0);
+            double e = 0.0;
+            for (int t0 = 0; t0 < d; t0 += 32) {
+                const int t = t0 + lane;
+                __syncwarp();
+                for (unsigned m = live; m; m &= m - 1u) {
+                    const int k = __ffs(m) - 1;
+                    const int64_t a = __shfl_sync(0xffffffffu, ra, k), b = __shfl_sync(0xffffffffu, rb, k);
+                    double v = 0.0;
+                    if (t < d) {
+                        const double df = __dsub_rn((double)x[a * d + t], (double)x[b * d + t]);
+                        v = __dmul_rn(df, df);
+                    }
+                    sq[wp][k][lane] = v;
+                }
+                __syncwarp();
+                if (jp >= 0) {
+                    const int tl = d - t0 < 32 ? d - t0 : 32;
+                    for (int u = 0; u < tl; ++u) e = __dadd_rn(e, sq[wp][lane][u]);
+                }
+            }
+            if (jp >= 0 && (bestj < 0 || key_less(e, i, j, best, i, bestj))) {
+                best = e;
+                bestj = j;
+            }
+        }
+        if (c > 0) {
+            rowd2[i] = best;
+            rowj[i] = bestj;
+        }
+    }
+}
+
 template <int EPL, int CW>
 __global__ void __launch_bounds__(256, 4) k_recheck_tc(const float *__restrict__ xs, int64_t n, int32_t d, int lists,
                                                        const float *__restrict__ tv, const int32_t *__restrict__ tj,
@@ -1038,7 +1102,8 @@ __global__ void __launch_bounds__(256, 4) k_recheck_tc(const float *__restrict__
                                                        int32_t *__restrict__ ovf, const int32_t *__restrict__ set_of,
                                                        const int32_t *__restrict__ setcnt, int32_t *counters,
                                                        int shard_rank, int shard_world,
-                                                       const int32_t *__restrict__ row_lists, float eps64) {
+                                                       const int32_t *__restrict__ row_lists, float eps64,
+                                                       unsigned int *__restrict__ rmin) {
     if (!mst_active(counters)) return;
     __shared__ int32_t bj_s[8][TC_TOPK];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -1047,19 +1112,126 @@ __global__ void __launch_bounds__(256, 4) k_recheck_tc(const float *__restrict__
     for (int64_t r = w0; r < n; r += nw)
         recheck_row<EPL, CW>(r, lane, xs, n, d, lists, tv, tj, tu, rsq, perm, compp, nmax_bits, eps_rep, mul32, add32, nsurv,
                              surv, rowj, ovf, set_of, setcnt, counters, bj_s[wib], shard_rank,
-                             shard_world, row_lists, eps64);
+                             shard_world, row_lists, eps64, rmin);
+}
+
+// ---- Rescan of the queued rows of one point set, by tiles: 32 queued rows
+// against 128 columns of the sweep's order, FP32 direct differences (4 x 4
+// pairs per thread), twice.  PASS 0 finds each row's FP32 minimum over the
+// columns of other components; PASS 1 records the columns within the error
+// margin of it as the recheck does, for k_exact_tc to key.  A row with more
+// than TC_SURV of them (exact ties) goes to k_rescan_tc.
+// Long rows far from the mean queue many rows: the sweep's bound carries 3 d
+// roundings of |y_i| |y_j|, at 3,279 x 1,558 (blobs at distance 230 from the
+// mean, points at 56 from each other) wider than the spread of the distances:
+// 7,791 rows in 4 rounds.  One block per row with a thread per column
+// (k_rescan_tc) read every row's line per lane and load: 104 ms there, 9 so.
+// Shorter rows queue few, and two launches more a round cost 30,011 x 20 2 %.
+constexpr int RS_R = 32, RS_C = 128, RS_D = 32, RS_MIN_D = 64;
+template <int PASS>
+__global__ void __launch_bounds__(256) k_rescan_tile(const float *__restrict__ xs, int64_t n, int32_t d,
+                                                     const int32_t *__restrict__ compp, const int32_t *__restrict__ ovf,
+                                                     unsigned int *__restrict__ rmin, float mul32, float add32,
+                                                     float eps64, const unsigned int *__restrict__ nmax_bits,
+                                                     int32_t *__restrict__ nsurv, int32_t *__restrict__ surv,
+                                                     const int32_t *__restrict__ counters) {
+    if (!mst_active(counters)) return;
+    const int nq = counters[MC_OVERFLOW];
+    if (nq == 0) return;
+    __shared__ __align__(16) float As[RS_D][RS_R + 4];
+    __shared__ __align__(16) float Bs[RS_D][RS_C + 4];
+    __shared__ int32_t sr[RS_R], sc[RS_R];
+    __shared__ float st[RS_R];
+    const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+    const int64_t ctiles = n / RS_C, items = (int64_t)((nq + RS_R - 1) / RS_R) * ctiles;      // (n: whole tiles)
+    for (int64_t w = blockIdx.x; w < items; w += gridDim.x) {
+        const int q0 = (int)(w / ctiles) * RS_R;
+        const int64_t col0 = (w % ctiles) * RS_C;
+        __syncthreads();
+        if (tid < RS_R) {
+            const int32_t r = q0 + tid < nq ? ovf[q0 + tid] : -1;
+            sr[tid] = r;
+            sc[tid] = r >= 0 ? compp[r] : -2;
+            if (PASS == 1 && r >= 0) {
+                float thr = __fadd_ru(__fmul_ru(__uint_as_float(rmin[r]), mul32), add32);
+                if (eps64 > 0.0f)
+                    thr = widen_f64(thr, __fmul_ru(2.0f * eps64, __fsqrt_ru(__uint_as_float(*nmax_bits))));
+                st[tid] = thr;
+            }
+        }
+        float acc[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = 0.0f;
+        for (int t0 = 0; t0 < d; t0 += RS_D) {
+            __syncthreads();
+            for (int e = tid; e < RS_R * RS_D; e += 256) {
+                const int r = e / RS_D, t = e % RS_D;
+                As[t][r] = sr[r] >= 0 && t0 + t < d ? xs[(int64_t)sr[r] * d + t0 + t] : 0.0f;
+            }
+#pragma unroll 4
+            for (int e = tid; e < RS_C * RS_D; e += 256) {
+                const int c = e / RS_D, t = e % RS_D;
+                Bs[t][c] = t0 + t < d ? xs[(col0 + c) * d + t0 + t] : 0.0f;
+            }
+            __syncthreads();
+#pragma unroll 8
+            for (int t = 0; t < RS_D; ++t) {
+                const float4 a4 = *reinterpret_cast<const float4 *>(&As[t][ty * 4]);
+                const float4 b4 = *reinterpret_cast<const float4 *>(&Bs[t][tx * 4]);
+                const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float df = __fsub_rn(a[i], b[j]);
+                        acc[i][j] = __fmaf_rn(df, df, acc[i][j]);
+                    }
+            }
+        }
+        int32_t cc[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) cc[j] = compp[col0 + tx * 4 + j];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int rr = ty * 4 + i;
+            const int32_t r = sr[rr], cr = sc[rr];
+            if (PASS == 0) {
+                float m = INFINITY;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (cc[j] >= 0 && cc[j] != cr) m = fminf(m, acc[i][j]);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                // (non-negative floats: their bits are in order)
+                if (tx == 0 && r >= 0 && m < INFINITY) atomicMin(rmin + r, __float_as_uint(m));
+            } else if (r >= 0) {
+                const float thr = st[rr];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (cc[j] >= 0 && cc[j] != cr && acc[i][j] <= thr) {
+                        const int q = atomicAdd(nsurv + r, 1);
+                        if (q < TC_SURV) surv[(int64_t)r * TC_SURV + q] = (int32_t)(col0 + tx * 4 + j);
+                    }
+            }
+        }
+    }
 }
 
 // Self-contained rescan of a queued row: FP32 direct differences give the
 // minimum m; every column within the FP32 error margin of m is keyed in FP64.
-// With independent sets only the row's own set is scanned.
+// With independent sets only the row's own set is scanned; tiled: only the
+// rows the tiles left over (more than TC_SURV columns in the margin).
 // Xe: the points the keys are taken from (FP64 input: X is their FP32 copy).
 template <class P>
 __global__ void __launch_bounds__(256) k_rescan_tc(const float *__restrict__ X, const P *__restrict__ Xe, int64_t n,
                                                    int32_t d,
                                                    const int32_t *__restrict__ comp, const int32_t *__restrict__ ovf,
+                                                   const int32_t *__restrict__ permp,
+                                                   const int32_t *__restrict__ nsurv,
                                                    const int32_t *__restrict__ set_of, const int64_t *__restrict__ offs,
-                                                   double mul, double add, float eps64,
+                                                   int tiled, double mul, double add, float eps64,
                                                    const unsigned int *__restrict__ nmax_bits,
                                                    double *__restrict__ rowd2, int32_t *__restrict__ rowj,
                                                    int32_t *counters) {
@@ -1069,7 +1241,8 @@ __global__ void __launch_bounds__(256) k_rescan_tc(const float *__restrict__ X, 
     __shared__ int32_t sj[256];
     const int nq = counters[MC_OVERFLOW];
     for (int q = blockIdx.x; q < nq; q += gridDim.x) {
-        const int64_t i = ovf[q];
+        if (tiled && nsurv[ovf[q]] <= TC_SURV) continue;
+        const int64_t i = permp[ovf[q]];
         const int32_t ci = comp[i];
         const float *xi = X + i * d;
         const int64_t j0 = set_of ? offs[set_of[i]] : 0, j1 = set_of ? offs[set_of[i] + 1] : n;
@@ -1194,6 +1367,7 @@ void TcScratch::carve(Arena &A, int64_t n, int32_t d, int splits_, int64_t n_pad
     kbuf = A.take<uint64_t>(n);
     compp = A.take<int32_t>(n_pad);
     nsurv = A.take<int32_t>(n_pad);
+    rmin = A.take<unsigned int>(n_pad);
     surv = A.take<int32_t>((size_t)n_pad * TC_SURV);
     tv = A.take<float>((size_t)lists * n_pad * TC_TOPK);
     tj = A.take<int32_t>((size_t)lists * n_pad * TC_TOPK);
@@ -1608,7 +1782,7 @@ cudaError_t tc_sweep_round(TcScratch &T, MstScratch &S, const float *X, int64_t 
     k_recheck_tc<EPLV, CWV><<<(unsigned)(rblocks < rcap ? rblocks : rcap), 256, 0, ISO_S(s)>>>(                        \
         T.xs, T.n_pad, d, T.lists, T.tv, T.tj, T.tu, T.rsq, T.permp, T.compp, T.nmax_bits, (float)(eps_rep * 1.0001),  \
         mul32, add32, T.nsurv, T.surv, S.rowj, S.ovf_rows, T.set_of, T.setcnt, S.counters, T.shard_rank,           \
-        T.shard_world, pruned ? T.nlists : nullptr, eps64)
+        T.shard_world, pruned ? T.nlists : nullptr, eps64, T.rmin)
     if (T.lists <= 4)
         {
         if (T.cw == 32) ISO_RECHECK_LAUNCH(1, 32);
@@ -1632,19 +1806,33 @@ cudaError_t tc_sweep_round(TcScratch &T, MstScratch &S, const float *X, int64_t 
 #undef ISO_RECHECK_LAUNCH
     const int64_t xblocks = ceil_div(T.n_pad, 256), xcap = (int64_t)num_sms() * 8;
     const unsigned xg = (unsigned)(xblocks < xcap ? xblocks : xcap);
-    if (T.f64) {
-        k_exact_tc<double><<<xg, 256, 0, ISO_S(s)>>>(T.x64, 1, T.n_pad, d, T.permp, T.nsurv, T.surv, S.rowd2, S.rowj,
-                                                     S.counters);
-        k_rescan_tc<double><<<(unsigned)(num_sms() * 4), 256, 0, ISO_S(s)>>>(
-            X, T.x64, n, d, S.comp, S.ovf_rows, T.set_of, T.offs, mul, add, eps64, T.nmax_bits, S.rowd2, S.rowj,
-            S.counters);
-    } else {
-        k_exact_tc<float><<<xg, 256, 0, ISO_S(s)>>>(T.xs, 0, T.n_pad, d, T.permp, T.nsurv, T.surv, S.rowd2, S.rowj,
-                                                    S.counters);
-        k_rescan_tc<float><<<(unsigned)(num_sms() * 4), 256, 0, ISO_S(s)>>>(
-            X, X, n, d, S.comp, S.ovf_rows, T.set_of, T.offs, mul, add, 0.0f, T.nmax_bits, S.rowd2, S.rowj,
-            S.counters);
+    const bool tiled = !T.set_of && d >= RS_MIN_D;
+    if (tiled) {
+        const unsigned tg = (unsigned)(num_sms() * 4);
+        k_rescan_tile<0><<<tg, 256, 0, ISO_S(s)>>>(T.xs, T.n_pad, d, T.compp, S.ovf_rows, T.rmin, mul32, add32, eps64,
+                                                   T.nmax_bits, T.nsurv, T.surv, S.counters);
+        k_rescan_tile<1><<<tg, 256, 0, ISO_S(s)>>>(T.xs, T.n_pad, d, T.compp, S.ovf_rows, T.rmin, mul32, add32, eps64,
+                                                   T.nmax_bits, T.nsurv, T.surv, S.counters);
     }
+    const bool wide = d >= EX_WIDE_MIN_D;
+    const unsigned wg = (unsigned)(2 * xblocks < xcap ? 2 * xblocks : xcap);
+#define ISO_EXACT(PT, XV, BY)                                                                                             \
+    (wide ? k_exact_wide<PT><<<wg, 128, 0, ISO_S(s)>>>(XV, BY, T.n_pad, d, T.permp, T.nsurv, T.surv, S.rowd2, S.rowj,      \
+                                                       S.counters)                                                        \
+          : k_exact_tc<PT><<<xg, 256, 0, ISO_S(s)>>>(XV, BY, T.n_pad, d, T.permp, T.nsurv, T.surv, S.rowd2, S.rowj,        \
+                                                     S.counters))
+    if (T.f64) {
+        ISO_EXACT(double, T.x64, 1);
+        k_rescan_tc<double><<<(unsigned)(num_sms() * 4), 256, 0, ISO_S(s)>>>(
+            X, T.x64, n, d, S.comp, S.ovf_rows, T.permp, T.nsurv, T.set_of, T.offs, tiled ? 1 : 0, mul, add, eps64, T.nmax_bits, S.rowd2,
+            S.rowj, S.counters);
+    } else {
+        ISO_EXACT(float, T.xs, 0);
+        k_rescan_tc<float><<<(unsigned)(num_sms() * 4), 256, 0, ISO_S(s)>>>(
+            X, X, n, d, S.comp, S.ovf_rows, T.permp, T.nsurv, T.set_of, T.offs, tiled ? 1 : 0, mul, add, 0.0f, T.nmax_bits, S.rowd2,
+            S.rowj, S.counters);
+    }
+#undef ISO_EXACT
     (void)status;
     return cudaGetLastError();
 }
