@@ -361,7 +361,7 @@ __device__ void init_search(SearchState *S, double phs, double phm, double wsum,
     S->stats[0] = phs; S->stats[1] = phm; S->stats[2] = wsum; S->stats[3] = wmin;
     S->stats[4] = psum; S->stats[5] = pmin; S->stats[6] = alpha0; S->stats[7] = beta0;
     S->have_lo = 0; S->have_hi = 0; S->done = 0; S->error = 0; S->passes = 0;
-    S->selected = 0; S->ik_bits = 0ull; S->beta = 0.0;
+    S->selected = 0; S->ik_bits = 0ull; S->beta = 0.0; S->ticket = 0;
     S->lane_lo = -1; S->mode = 0; S->cand_passes = 0; S->ncand = 0u;
     const double DMAX = 1.7976931348623157e308;
     double b0 = (isfinite(beta0) && beta0 > 0.0) ? beta0 : 1.0;
@@ -862,22 +862,26 @@ __global__ void __launch_bounds__(256) k_cand_hist(DpArgs A, SearchState *S, con
     }
 }
 
-// One block: the next pass's thresholds (lane 0 = lo), or the switch to the
-// 33-ary bit search already written by k_search_update.
-__global__ void __launch_bounds__(1024) k_cand_select(SearchState *S, uint32_t *__restrict__ hist) {
-    __shared__ unsigned int pre[CAND_BUCKETS];
+// No critical ratio lies inside the bracket: in lo's state no decision
+// changes before hi, so beta is hi but for the comparisons' rounding.  The
+// doubles just below hi (1, 2, 4, ... steps) close the bracket, usually in
+// one pass (the 33-ary bit search it was left to took up to 11 more).
+__device__ __forceinline__ int below_hi(double *t, int used, unsigned long long lo, unsigned long long hi) {
+    for (unsigned long long g = 1ull; used < DP_LANES - 1 && g < hi - lo; g <<= 1) t[used++] = bitsd(hi - g);
+    return used;
+}
+
+// One block of NT threads: the next pass's thresholds (lane 0 = lo), or the
+// switch to the 33-ary bit search already written by search_update.  hist:
+// the counted ratios per bucket, zeroed on the way out; pre: CAND_BUCKETS
+// words of scratch; nc, cand: the number of counted ratios and the first ones.
+template <int NT>
+__device__ void cand_select_block(SearchState *S, uint32_t *hist, unsigned int *pre, unsigned int nc,
+                                  const unsigned long long *cand) {
     __shared__ unsigned int warp_sum[32];
-    __shared__ int active;
     const int tid = threadIdx.x;
-    if (tid == 0) active = cand_active(S) ? 1 : 0;
-    __syncthreads();
-    if (!active) {
-        if (tid == 0 && !S->done) S->mode = 1;       // k_search_update's bit-search thresholds stand
-        for (int j = tid; j < CAND_BUCKETS; j += blockDim.x) hist[j] = 0u;
-        return;
-    }
-    // inclusive prefix sums of the buckets: 4 per thread, then across threads
-    constexpr int PER = CAND_BUCKETS / 1024;
+    // inclusive prefix sums of the buckets: PER per thread, then across threads
+    constexpr int PER = CAND_BUCKETS / NT;
     unsigned int loc[PER], run = 0;
 #pragma unroll
     for (int q = 0; q < PER; ++q) { run += hist[tid * PER + q]; loc[q] = run; }
@@ -891,7 +895,7 @@ __global__ void __launch_bounds__(1024) k_cand_select(SearchState *S, uint32_t *
     if (lane == 31) warp_sum[wp] = x;
     __syncthreads();
     if (wp == 0) {
-        unsigned int z = warp_sum[lane];
+        unsigned int z = lane < NT / 32 ? warp_sum[lane] : 0u;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const unsigned int y = __shfl_up_sync(0xffffffffu, z, o);
@@ -904,12 +908,10 @@ __global__ void __launch_bounds__(1024) k_cand_select(SearchState *S, uint32_t *
 #pragma unroll
     for (int q = 0; q < PER; ++q) pre[tid * PER + q] = before + loc[q];
     __syncthreads();
-    for (int j = tid; j < CAND_BUCKETS; j += blockDim.x) hist[j] = 0u;     // ready for the next pass
+    for (int j = tid; j < CAND_BUCKETS; j += NT) hist[j] = 0u;     // ready for the next pass
     if (tid != 0) return;
     const unsigned long long lo = S->lo_bits, hi = S->hi_bits;
     const unsigned int m = pre[CAND_BUCKETS - 1];
-    const unsigned int nc = S->ncand;
-    S->ncand = 0u;
     double t[DP_LANES];
     t[0] = bitsd(lo);
     int used = 1;
@@ -918,12 +920,11 @@ __global__ void __launch_bounds__(1024) k_cand_select(SearchState *S, uint32_t *
         for (int q = 1; q < DP_LANES; ++q) t[q] = bitsd(lo + (unsigned long long)q < hi ? lo + q : hi);
         used = DP_LANES;
     } else if (m == 0u) {
-        S->mode = 1;                                  // nothing to aim at: bit search
-        return;
+        used = below_hi(t, used, lo, hi);
     } else if (nc <= (unsigned)CAND_EXACT) {
         // each remaining critical ratio and its neighbouring doubles
         for (unsigned q = 0; q < nc && used + 3 <= DP_LANES; ++q) {
-            const unsigned long long b = S->cand[q];
+            const unsigned long long b = cand[q];
             const unsigned long long c[3] = {b - 1ull, b, b + 1ull};
             for (int r = 0; r < 3; ++r)
                 if (c[r] > lo && c[r] < hi) t[used++] = bitsd(c[r]);
@@ -949,6 +950,179 @@ __global__ void __launch_bounds__(1024) k_cand_select(SearchState *S, uint32_t *
     S->cand_passes += 1;
 }
 
+__global__ void __launch_bounds__(1024) k_cand_select(SearchState *S, uint32_t *__restrict__ hist) {
+    __shared__ unsigned int pre[CAND_BUCKETS];
+    __shared__ int active;
+    __shared__ unsigned int nc;
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        active = cand_active(S) ? 1 : 0;
+        nc = S->ncand;
+        if (active) S->ncand = 0u;
+    }
+    __syncthreads();
+    if (!active) {
+        if (tid == 0 && !S->done) S->mode = 1;       // search_update's bit-search thresholds stand
+        for (int j = tid; j < CAND_BUCKETS; j += blockDim.x) hist[j] = 0u;
+        return;
+    }
+    cand_select_block<1024>(S, hist, pre, nc, S->cand);
+}
+
+// ---- Trees of at most SM_MAX_N vertices: one block per threshold evaluates
+// Algorithm 1 on the whole tree out of shared memory, level by level from the
+// deepest, in BFS order (a vertex's children are then contiguous).  A level
+// costs a barrier and a few shared-memory round trips (about 0.3 us) where a
+// step of the walks through global memory costs 2.5 us: 4,898 points (depth
+// 116) 0.28 ms a pass -> 0.04.  The block that finishes last updates the
+// search and picks the next thresholds, so a pass is one launch.  States go
+// out by [threshold][BFS position].
+constexpr int SM_THREADS = 512;
+constexpr int SM_MAX_N = 12288;       // 17 bytes a vertex: 204 KB of shared memory
+constexpr int SM_MIN_SMEM = 2 * CAND_BUCKETS * (int)sizeof(uint32_t);
+inline int sm_smem(int64_t n) { return (int)(n * 17 > SM_MIN_SMEM ? n * 17 : SM_MIN_SMEM); }
+
+struct SmallTree {
+    int32_t n;
+    const int32_t *order;                       // vertex of a BFS position
+    double *omega, *p, *phi;                    // by BFS position
+    int32_t *c0, *nc;                           // first child's position, number of children
+    int32_t *lstart;                            // first position of a level
+    uint8_t *dec;                               // [DP_LANES][n]
+    double *wh, *ph;
+    double *rat;                                // by vertex
+};
+
+__global__ void k_small_setup(SmallTree A, const int32_t *__restrict__ ch_off, const int32_t *__restrict__ ch_list,
+                              const int32_t *__restrict__ bfs_pos, const int32_t *__restrict__ depth,
+                              const double *__restrict__ phi, const double *__restrict__ omega,
+                              const double *__restrict__ p) {
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= A.n) return;
+    const int32_t v = A.order[q];
+    A.omega[q] = omega[v];
+    A.p[q] = p ? p[v] : 0.0;
+    A.phi[q] = phi[v];
+    const int32_t a = ch_off[v], b = ch_off[v + 1];
+    A.nc[q] = b - a;
+    A.c0[q] = b > a ? bfs_pos[ch_list[a]] : 0;
+    if (q == 0 || depth[A.order[q - 1]] != depth[v]) A.lstart[depth[v]] = q;
+}
+
+__global__ void __launch_bounds__(SM_THREADS) k_dp_small(SmallTree A, SearchState *S, int32_t k, int last, int final_pass,
+                                                         uint32_t *st) {
+    if (!final_pass && S->done) return;
+    if (final_pass && (S->final_lane >= 0 || blockIdx.x != 0)) return;      // (k_final_from_lane serves)
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    const int n = A.n, tid = threadIdx.x, t = blockIdx.x;
+    double *W = reinterpret_cast<double *>(sm_raw), *P = W + n;
+    uint8_t *Dc = reinterpret_cast<uint8_t *>(P + n);
+    __shared__ int scuts, slast;
+    if (tid == 0) scuts = 0;
+    const double N = final_pass ? S->beta : S->thr[t];
+    uint8_t *gd = A.dec + (size_t)t * n;
+    double *gw = A.wh + (size_t)t * n, *gp = A.ph + (size_t)t * n;
+    int cuts = 0;
+    struct Vtx {
+        double w, p, f;
+        int c0, nc;
+    };
+    auto load = [&](int q) { return Vtx{A.omega[q], A.p[q], A.phi[q], A.c0[q], A.nc[q]}; };
+    auto decide = [&](int q, const Vtx &x) {
+        double w = x.w, pv = x.p;
+        for (int c = x.c0 + x.nc - 1; c >= x.c0; --c) {        // siblings in descending index
+            pv = __dadd_rn(pv, P[c]);                          // (a child that did not join left its edge's phi there)
+            if (Dc[c] == DEC_JOIN) w = __dadd_rn(w, W[c]);
+        }
+        const double fe = q > 0 ? x.f : 0.0;
+        const double nw = __dmul_rn(N, w), fp = __dadd_rn(fe, pv);
+        uint8_t d;
+        if (fp <= nw) {
+            d = DEC_CUT;
+            ++cuts;
+            if (final_pass) A.rat[A.order[q]] = __ddiv_rn(fp, w);
+        } else if (q > 0 && __dsub_rn(pv, fe) < nw) {
+            d = DEC_JOIN;
+        } else {
+            d = DEC_DISCARD;
+        }
+        Dc[q] = d;
+        W[q] = w;
+        P[q] = d == DEC_JOIN ? pv : fe;
+        gd[q] = d;
+        gw[q] = w;
+        gp[q] = pv;
+    };
+    // the next level's first vertices are on their way while a level is decided
+    int l = S->max_depth;
+    int s0 = A.lstart[l], e0 = n, s1 = l > 0 ? A.lstart[l - 1] : 0;
+    Vtx cur{}, nxt{};
+    if (s0 + tid < e0) cur = load(s0 + tid);
+    __syncthreads();
+    for (; l >= 0; --l) {
+        const int s2 = l > 1 ? A.lstart[l - 2] : 0;
+        if (l > 0 && s1 + tid < s0) nxt = load(s1 + tid);
+        if (s0 + tid < e0) decide(s0 + tid, cur);
+        for (int q = s0 + tid + SM_THREADS; q < e0; q += SM_THREADS) decide(q, load(q));
+        __syncthreads();
+        cur = nxt;
+        e0 = s0;
+        s0 = s1;
+        s1 = s2;
+    }
+    for (int o = 16; o > 0; o >>= 1) cuts += __shfl_xor_sync(0xffffffffu, cuts, o);
+    if ((tid & 31) == 0 && cuts) atomicAdd(&scuts, cuts);
+    __threadfence();
+    __syncthreads();
+    if (final_pass) return;
+    if (tid == 0) {
+        S->cnt[t] = scuts;
+        __threadfence();
+        slast = atomicAdd(&S->ticket, 1) == DP_LANES - 1;
+    }
+    __syncthreads();
+    if (!slast) return;
+    // ---- the last block: bracket, critical ratios in lo's state, thresholds
+    __shared__ unsigned int snc;
+    __shared__ unsigned long long scand[CAND_EXACT];
+    __shared__ int sact, sL;
+    __shared__ unsigned long long slo, shi;
+    uint32_t *hist = reinterpret_cast<uint32_t *>(sm_raw);
+    unsigned int *pre = reinterpret_cast<unsigned int *>(sm_raw) + CAND_BUCKETS;
+    __threadfence();
+    if (tid == 0) {
+        S->ticket = 0;
+        search_update(S, k, last, st);
+        sact = cand_active(S) ? 1 : 0;
+        if (!sact && !S->done) S->mode = 1;                    // the bit-search thresholds stand
+        sL = S->lane_lo;
+        slo = S->lo_bits;
+        shi = S->hi_bits;
+        snc = 0u;
+    }
+    for (int j = tid; j < CAND_BUCKETS; j += SM_THREADS) hist[j] = 0u;
+    __syncthreads();
+    if (!sact) return;
+    const unsigned long long lo = slo, hi = shi;
+    const double inv_w = (double)CAND_BUCKETS / (double)(hi - lo);
+    auto add = [&](double c) {
+        const unsigned long long b = dbits(c);
+        if (!(c > 0.0) || b <= lo || b >= hi) return;
+        atomicAdd(hist + cand_bucket(b, lo, inv_w), 1u);
+        const unsigned q = atomicAdd(&snc, 1u);
+        if (q < (unsigned)CAND_EXACT) scand[q] = b;
+    };
+    const double *lw = A.wh + (size_t)sL * n, *lp = A.ph + (size_t)sL * n;
+    for (int q = tid; q < n; q += SM_THREADS) {
+        const double w = ld_cg_f64(lw + q), pv = ld_cg_f64(lp + q);
+        const double fe = q > 0 ? A.phi[q] : 0.0;
+        add(__ddiv_rn(__dadd_rn(fe, pv), w));
+        if (q > 0) add(__ddiv_rn(__dsub_rn(pv, fe), w));
+    }
+    __syncthreads();
+    cand_select_block<SM_THREADS>(S, hist, pre, snc, scand);
+}
+
 // After the search (one tree): the lane of the last pass that evaluated beta
 // itself, if any.  Its decisions and omega-hat / p-hat are those of the
 // final call of Algorithm 1 at beta, so k_final_from_lane copies them to
@@ -963,14 +1137,14 @@ __global__ void k_final_lane(SearchState *S) {
 }
 
 __global__ void k_final_from_lane(const SearchState *__restrict__ S, const int32_t *__restrict__ parent,
-                                  const double *__restrict__ phi, const int32_t *__restrict__ slot, int64_t n,
-                                  uint8_t *__restrict__ dec, const double *__restrict__ wh,
+                                  const double *__restrict__ phi, const int32_t *__restrict__ slot, int64_t sv,
+                                  int64_t sl, int64_t n, uint8_t *__restrict__ dec, const double *__restrict__ wh,
                                   const double *__restrict__ ph, double *__restrict__ rat) {
     const int L = S->final_lane;
     if (L < 0) return;
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n) return;
-    const size_t s0 = (size_t)slot[v] * DP_LANES, vl = s0 + L;
+    const size_t s0 = (size_t)slot[v] * sv, vl = s0 + (size_t)L * sl;
     const uint8_t d = dec[vl];
     dec[s0] = d;
     if (d == DEC_CUT) {
@@ -1061,8 +1235,7 @@ __global__ void __launch_bounds__(256) k_cand_select_sets(SearchState *SS, int32
         for (int q = 1; q < DP_LANES; ++q) t[q] = bitsd(lo + (unsigned long long)q < hi ? lo + q : hi);
         used = DP_LANES;
     } else if (m == 0u) {
-        S->mode = 1;
-        return;
+        used = below_hi(t, used, lo, hi);
     } else if (nc <= (unsigned)CAND_EXACT) {
         for (unsigned q = 0; q < nc && used + 3 <= DP_LANES; ++q) {
             const unsigned long long c0 = S->cand[q];
@@ -1102,10 +1275,12 @@ __global__ void k_search_update_sets(SearchState *SS, const int32_t *__restrict_
 __global__ void k_sets_left_init(uint32_t *left, int32_t nsets) { *left = (uint32_t)nsets; }
 
 // ------------------------------------------------------------ labels
-__global__ void k_head_init(const uint8_t *__restrict__ dec, const int32_t *__restrict__ slot,
+// (one tree: the state of vertex v at the last pass's lane L is at slot[v] sv
+// + L sl; the final decisions are lane 0's)
+__global__ void k_head_init(const uint8_t *__restrict__ dec, const int32_t *__restrict__ slot, int64_t sv,
                             const int32_t *__restrict__ parent, int64_t n, int32_t *__restrict__ head) {
     int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < n) head[v] = dec[(size_t)(slot ? slot[v] : (int32_t)v) * DP_LANES] == DEC_JOIN ? parent[v] : (int32_t)v;
+    if (v < n) head[v] = dec[(size_t)(slot ? slot[v] : (int32_t)v) * sv] == DEC_JOIN ? parent[v] : (int32_t)v;
 }
 
 __global__ void k_head_jump(const int32_t *__restrict__ hin, int32_t *__restrict__ hout, int64_t n) {
@@ -1113,13 +1288,13 @@ __global__ void k_head_jump(const int32_t *__restrict__ hin, int32_t *__restrict
     if (v < n) hout[v] = hin[hin[v]];
 }
 
-__global__ void k_cut_flags(const uint8_t *__restrict__ dec, const int32_t *__restrict__ slot,
+__global__ void k_cut_flags(const uint8_t *__restrict__ dec, const int32_t *__restrict__ slot, int64_t sv,
                             const int32_t *__restrict__ bfs_pos, int64_t n, int32_t *__restrict__ cflag) {
     int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < n) cflag[n - 1 - bfs_pos[v]] = dec[(size_t)(slot ? slot[v] : (int32_t)v) * DP_LANES] == DEC_CUT ? 1 : 0;
+    if (v < n) cflag[n - 1 - bfs_pos[v]] = dec[(size_t)(slot ? slot[v] : (int32_t)v) * sv] == DEC_CUT ? 1 : 0;
 }
 
-__global__ void k_labels(const uint8_t *__restrict__ dec, const int32_t *__restrict__ slot,
+__global__ void k_labels(const uint8_t *__restrict__ dec, const int32_t *__restrict__ slot, int64_t sv,
                          const int32_t *__restrict__ bfs_pos,
                          const int32_t *__restrict__ head, const int32_t *__restrict__ cidx,
                          const double *__restrict__ rat, int64_t n, int32_t k, int32_t *__restrict__ labels,
@@ -1127,11 +1302,11 @@ __global__ void k_labels(const uint8_t *__restrict__ dec, const int32_t *__restr
     int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n) return;
     int32_t h = head[v];
-    int32_t c = dec[(size_t)slot[h] * DP_LANES] == DEC_CUT ? cidx[n - 1 - bfs_pos[h]] : -1;
+    int32_t c = dec[(size_t)slot[h] * sv] == DEC_CUT ? cidx[n - 1 - bfs_pos[h]] : -1;
     int32_t lab = (c >= 0 && c < k) ? c : -1;
     labels[v] = lab;
     residual[v] = lab < 0 ? 1 : 0;
-    if (dec[(size_t)slot[v] * DP_LANES] == DEC_CUT) {
+    if (dec[(size_t)slot[v] * sv] == DEC_CUT) {
         int32_t cv = cidx[n - 1 - bfs_pos[v]];
         if (cv < k) {
             atomicMax(&S->ik_bits, dbits(rat[v]));
@@ -1326,38 +1501,94 @@ cudaError_t tree_search_and_label(TreeScratch &S, const double *phi_par, const d
     cudaError_t e;
     k_stats_part<<<STATS_BLOCKS, 256, 0, ISO_S(s)>>>(T.parent, phi_par, omega, p, n, S.spart, S.status);
     k_stats_final<<<1, STATS_BLOCKS, 0, ISO_S(s)>>>(S.spart, n, S.search);
-    k_phi_slots<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(T.ch_list, phi_par, n - 1, S.phis);
-    DpArgs A{n, T.parent, T.ch_off, T.ch_list, T.leaves, phi_par, omega, p, T.slot, S.phis};
-    const unsigned grid = (unsigned)(num_sms() * 8);
-    if ((e = cudaMemsetAsync(S.hist, 0, sizeof(uint32_t) * CAND_BUCKETS, s))) return e;
-    for (int pass = 0; pass < DP_TREE_PASSES; ++pass) {
-        if ((e = cudaMemsetAsync(S.done, 0, sizeof(int32_t) * n, s))) return e;
-        k_dp_pass<<<grid, 256, 0, ISO_S(s)>>>(A, S.search, S.dec, S.wh, S.ph, S.done, S.rat, 0);
-        k_search_update<<<1, 32, 0, ISO_S(s)>>>(S.search, k, pass == DP_TREE_PASSES - 1, S.status);
-        if (pass + 1 < DP_TREE_PASSES) {
+    // The passes end when the device says so: it is asked after the first few
+    // passes and every few after that (most searches take 2 to 4; the rest of
+    // the 22 would be launches that return at once, 0.2 to 0.4 ms of them).
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if ((e = cudaStreamIsCapturing(s, &cs))) return e;
+    const bool ask = cs == cudaStreamCaptureStatusNone;
+    auto finished = [&](bool *fin) -> cudaError_t {
+        int done = 0;
+        cudaError_t r = cudaMemcpyAsync(&done, &S.search->done, sizeof(int), cudaMemcpyDeviceToHost, s);
+        if (!r) r = cudaStreamSynchronize(s);
+        *fin = done != 0;
+        return r;
+    };
+    const bool small = n >= 2 && n <= SM_MAX_N;
+    const int32_t *slot = T.slot;
+    int64_t sv = DP_LANES, sl = 1;
+    if (small) {
+        // (the orientation's buffers are free by now)
+        SmallTree A;
+        A.n = (int32_t)n;
+        A.order = S.ib;
+        A.omega = reinterpret_cast<double *>(S.ssz);
+        A.p = reinterpret_cast<double *>(S.sx);
+        A.phi = reinterpret_cast<double *>(S.kbuf);
+        A.c0 = S.rev;
+        A.nc = S.succ;
+        A.lstart = S.succ2;
+        A.dec = S.dec;
+        A.wh = S.wh;
+        A.ph = S.ph;
+        A.rat = S.rat;
+        const int smem = sm_smem(n);
+        static bool attr = false;
+        if (!attr) {
+            if ((e = cudaFuncSetAttribute(k_dp_small, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_smem(SM_MAX_N))))
+                return e;
+            attr = true;
+        }
+        k_small_setup<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(A, T.ch_off, T.ch_list, T.bfs_pos, T.depth, phi_par, omega, p);
+        for (int pass = 0; pass < DP_TREE_PASSES; ++pass) {
+            k_dp_small<<<DP_LANES, SM_THREADS, smem, ISO_S(s)>>>(A, S.search, k, pass == DP_TREE_PASSES - 1, 0, S.status);
+            bool fin = false;
+            if (ask && pass % 3 == 2 && pass + 1 < DP_TREE_PASSES && (e = finished(&fin))) return e;
+            if (fin) break;
+        }
+        slot = T.bfs_pos;
+        sv = 1;
+        sl = n;
+        k_final_lane<<<1, 32, 0, ISO_S(s)>>>(S.search);
+        k_final_from_lane<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.search, T.parent, phi_par, slot, sv, sl, n, S.dec, S.wh,
+                                                               S.ph, S.rat);
+        k_dp_small<<<1, SM_THREADS, smem, ISO_S(s)>>>(A, S.search, k, 0, 1, S.status);
+    } else {
+        k_phi_slots<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(T.ch_list, phi_par, n - 1, S.phis);
+        DpArgs A{n, T.parent, T.ch_off, T.ch_list, T.leaves, phi_par, omega, p, T.slot, S.phis};
+        const unsigned grid = (unsigned)(num_sms() * 8);
+        if ((e = cudaMemsetAsync(S.hist, 0, sizeof(uint32_t) * CAND_BUCKETS, s))) return e;
+        for (int pass = 0; pass < DP_TREE_PASSES; ++pass) {
+            if ((e = cudaMemsetAsync(S.done, 0, sizeof(int32_t) * n, s))) return e;
+            k_dp_pass<<<grid, 256, 0, ISO_S(s)>>>(A, S.search, S.dec, S.wh, S.ph, S.done, S.rat, 0);
+            k_search_update<<<1, 32, 0, ISO_S(s)>>>(S.search, k, pass == DP_TREE_PASSES - 1, S.status);
+            if (pass + 1 == DP_TREE_PASSES) break;
+            bool fin = false;
+            if (ask && pass >= 1 && (e = finished(&fin))) return e;
+            if (fin) break;
             // the next pass's thresholds from the critical ratios in lo's state
             k_cand_hist<<<grid, 256, 0, ISO_S(s)>>>(A, S.search, S.wh, S.ph, S.hist);
             k_cand_select<<<1, 1024, 0, ISO_S(s)>>>(S.search, S.hist);
         }
+        // Final call of Algorithm 1 at beta: Cut, eta and the set ratios (from the
+        // last pass's lane at beta when it has one, else one more pass)
+        k_final_lane<<<1, 32, 0, ISO_S(s)>>>(S.search);
+        k_final_from_lane<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.search, T.parent, phi_par, slot, sv, sl, n, S.dec, S.wh,
+                                                               S.ph, S.rat);
+        if ((e = cudaMemsetAsync(S.done, 0, sizeof(int32_t) * n, s))) return e;
+        k_dp_pass<<<grid, 256, 0, ISO_S(s)>>>(A, S.search, S.dec, S.wh, S.ph, S.done, S.rat, 1);
     }
-    // Final call of Algorithm 1 at beta: Cut, eta and the set ratios (from the
-    // last pass's lane at beta when it has one, else one more pass)
-    k_final_lane<<<1, 32, 0, ISO_S(s)>>>(S.search);
-    k_final_from_lane<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.search, T.parent, phi_par, T.slot, n, S.dec, S.wh, S.ph,
-                                                           S.rat);
-    if ((e = cudaMemsetAsync(S.done, 0, sizeof(int32_t) * n, s))) return e;
-    k_dp_pass<<<grid, 256, 0, ISO_S(s)>>>(A, S.search, S.dec, S.wh, S.ph, S.done, S.rat, 1);
     // Algorithm 4: eta by pointer jumping, exclusive scan over Cut.
-    k_head_init<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, T.slot, T.parent, n, S.head);
+    k_head_init<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, slot, sv, T.parent, n, S.head);
     int32_t *ha = S.head, *hb = S.head2;
     const int Ln = log2_ceil(n) + 1;
     for (int it = 0; it < Ln; ++it) {
         k_head_jump<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(ha, hb, n);
         int32_t *t = ha; ha = hb; hb = t;
     }
-    k_cut_flags<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, T.slot, T.bfs_pos, n, S.cflag);
+    k_cut_flags<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, slot, sv, T.bfs_pos, n, S.cflag);
     if ((e = exclusive_scan_i32(S.cflag, S.cidx, n, S.tmp32, s))) return e;
-    k_labels<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, T.slot, T.bfs_pos, ha, S.cidx, S.rat, n, k, labels, residual, S.search);
+    k_labels<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, slot, sv, T.bfs_pos, ha, S.cidx, S.rat, n, k, labels, residual, S.search);
     k_finish<<<1, 32, 0, ISO_S(s)>>>(S.search, k, i_k, S.status);
     return cudaGetLastError();
 }
@@ -1400,14 +1631,14 @@ cudaError_t tree_search_and_label_sets(TreeScratch &S, int32_t nsets, const int6
     }
     if ((e = cudaMemsetAsync(S.done, 0, sizeof(int32_t) * n, s))) return e;
     k_dp_pass_sets<<<grid, 256, 0, ISO_S(s)>>>(A, S.search, SS, vset, S.dec, S.wh, S.ph, S.done, S.rat, 1, left);
-    k_head_init<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, nullptr, T.parent, n, S.head);
+    k_head_init<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, nullptr, DP_LANES, T.parent, n, S.head);
     int32_t *ha = S.head, *hb = S.head2;
     const int Ln = log2_ceil(n) + 1;
     for (int it = 0; it < Ln; ++it) {
         k_head_jump<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(ha, hb, n);
         int32_t *t = ha; ha = hb; hb = t;
     }
-    k_cut_flags<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, nullptr, T.bfs_pos, n, S.cflag);
+    k_cut_flags<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, nullptr, DP_LANES, T.bfs_pos, n, S.cflag);
     if ((e = exclusive_scan_i32(S.cflag, S.cidx, n, S.tmp32, s))) return e;
     k_labels_sets<<<blocks_for(nv), TPB, 0, ISO_S(s)>>>(S.dec, T.bfs_pos, ha, S.cidx, S.rat, nv, vset, offs, ks, labels,
                                                         residual, SS);

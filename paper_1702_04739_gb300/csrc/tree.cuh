@@ -37,6 +37,7 @@ struct SearchState {
     int cand_passes;          // passes that took their thresholds from critical ratios
     unsigned int ncand;       // critical ratios inside the bracket (this pass)
     unsigned long long cand[CAND_EXACT];
+    int ticket;               // blocks of a pass that are done (small trees)
     int final_lane;           // lane of the last pass whose threshold is beta (-1: none; one tree)
 };
 
