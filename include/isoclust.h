@@ -449,7 +449,7 @@ double isoclust_last_omega_gram_ms(int64_t *blocks, int64_t *direct_pairs);
 isoclust_status isoclust_set_sweep_variant(int32_t variant);
 
 /* The sweep variant of the last minimum-spanning-tree build on this host
- * thread (0..3), or -1 when none ran (FP32/FP64 sweep). */
+ * thread (0..3), or -1 when none ran (FP32/FP64 sweep, stored distances). */
 int32_t isoclust_last_sweep_variant(void);
 
 /* How the last isoclust_cluster_batched / _batched_detail call on this

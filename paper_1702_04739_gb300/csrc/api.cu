@@ -431,6 +431,12 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     TC.f64 = dtype == ISOCLUST_F64 && o.precision == ISOCLUST_PREC_AUTO && o.spin_limit == 0 && !TC.stall_test &&
              tc_supported();
     const bool tc_any = use_tc || TC.f64;
+    // a small set's rounds on stored distances; whoever asks for the
+    // tensor-core sweep (precision, variant, pruning, a limit on its waits)
+    // gets it
+    const bool dist = tc_any && !sh && o.precision == ISOCLUST_PREC_AUTO && o.spin_limit == 0 && !TC.stall_test &&
+                      tc_forced_variant() < 0 && prune_mode() != 1 && mst_dist_wanted(n, d, dtype);
+    float *dmat = nullptr;
     const int tsplits = tc_any ? tc_splits(n) : 1;
     if (sh) {
         // the sharded work: the tensor-core sweep and the symmetric omega sweep
@@ -479,6 +485,7 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
         *status = A.take<uint32_t>(4);
         M.carve(A, n, splits);
         if (tc_any) TC.carve(A, n, d, tsplits_used, 0, 1, tlists);
+        if (dist) dmat = (float *)A.take<unsigned char>(mst_dist_bytes(n));
         if (weights64) P.sym = (void *)A.take<unsigned char>(weights64_bytes(n, o.alpha != 0.0));
         if (need_labels) {
             TS.carve(A, n);
@@ -536,7 +543,13 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     }
 
     // Section 2.2 steps 1-2: minimum spanning tree
-    ISO_CUDA(mst_build(M, X, n, d, dtype, fp64_sweep, status, s, tc_used ? &TC : nullptr, 1, 0, sh));
+    const bool dist_used = dist && tc_used;
+    if (dist_used) {
+        tc_clear_last_variant();
+        ISO_CUDA(mst_build_dist(M, TC, dmat, X, n, d, dtype, TC.scale_exp, status, s));
+    } else {
+        ISO_CUDA(mst_build(M, X, n, d, dtype, fp64_sweep, status, s, tc_used ? &TC : nullptr, 1, 0, sh));
+    }
     const bool mst_pruned = TC.prune && TC.prune_ready;     // (the omega screen re-prepares TC later)
     unsigned long long mst_swept = 0;
     if (mst_pruned) {
@@ -647,7 +660,7 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     g_prof_cnt[2] = ss.passes + (need_labels ? 1 : 0);
     g_prof_cnt[3] = ss.max_depth;
     g_prof_mst_tiles[0] = g_prof_mst_tiles[1] = 0;
-    if (tc_used) {
+    if (tc_used && !dist_used) {
         const int64_t nt = TC.n_pad / 128;
         g_prof_mst_tiles[1] = (int64_t)cnt[MC_ROUNDS] * nt * nt;
         g_prof_mst_tiles[0] = g_prof_mst_tiles[1];

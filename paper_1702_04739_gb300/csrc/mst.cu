@@ -602,6 +602,11 @@ cudaError_t mst_build(MstScratch &S, const void *X, int64_t n, int32_t d, int dt
     return cudaGetLastError();
 }
 
+cudaError_t mst_component_minima(MstScratch &S, int64_t n, cudaStream_t s) {
+    k_cmin_d2<<<round_grid(n), TPB, 0, ISO_S(s)>>>(S.comp, S.rowd2, S.rowj, n, S.cd2, S.counters);
+    return cudaGetLastError();
+}
+
 cudaError_t nn_sweep(MstScratch &S, const void *X, int64_t n, int32_t d, int dtype, bool sweep_fp64,
                      uint32_t *status, cudaStream_t s, TcScratch *tc) {
     k_mst_init<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.comp, n, 1, S.counters);

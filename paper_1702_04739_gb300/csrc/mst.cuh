@@ -172,6 +172,20 @@ cudaError_t mst_build(MstScratch &S, const void *X, int64_t n, int32_t d, int dt
                       uint32_t *status, cudaStream_t s, TcScratch *tc = nullptr, int32_t target = 1,
                       int64_t max_n = 0, const Shard *sh = nullptr);
 
+// ---- stored distances (mst_dist.cu): one set whose FP32 distance matrix
+// (n^2 words in D) is formed once and read by every round.  TC gives the
+// buffers of the long rows' keys.
+size_t mst_dist_bytes(int64_t n);
+bool mst_dist_wanted(int64_t n, int32_t d, int dtype);
+cudaError_t mst_build_dist(MstScratch &S, TcScratch &T, float *D, const void *X, int64_t n, int32_t d, int dtype,
+                           int scale_exp, uint32_t *status, cudaStream_t s);
+// FP64 keys of the columns listed per row (T.nsurv, T.surv by point, T.permp
+// the identity) and of the rows listed for a rescan, into S.rowd2 / rowj
+cudaError_t tc_key_rows(TcScratch &T, MstScratch &S, const float *X, int64_t n, int32_t d, double mul, double add,
+                        cudaStream_t s);
+// S.cd2: per component the smallest of its rows' keys
+cudaError_t mst_component_minima(MstScratch &S, int64_t n, cudaStream_t s);
+
 // Nearest-neighbour d2 of every row (exact key), one Boruvka-style sweep with
 // every point its own component.  Result in S.rowd2 / S.rowj.
 cudaError_t nn_sweep(MstScratch &S, const void *X, int64_t n, int32_t d, int dtype, bool sweep_fp64,

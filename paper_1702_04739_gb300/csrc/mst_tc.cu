@@ -1030,24 +1030,28 @@ __global__ void __launch_bounds__(256) k_exact_tc(const P *__restrict__ x, int b
     }
 }
 
-// The same for long rows: a warp keys one column of each of its 32 rows at a
+// The same for long rows: a warp keys one column of each of its 8 rows at a
 // time.  The squares of 32 dimensions are formed by the lanes, a dimension
-// each (whole lines of the rows), and handed over in shared memory; each lane
-// then adds its own row's in order.  (A thread per row reads a line per lane
-// and load: 1.0 ms a round at 3,279 x 1,558.)
-constexpr int EX_WIDE_MIN_D = 256;
+// each (whole lines of the rows, the next ones on their way), and handed over
+// in shared memory; 8 lanes then add their own row's in order.  Bound by the
+// latency of that chain of additions: 180 x 1,500 0.7 ms a round with 32 rows
+// to a warp and one load in flight, 3,279 x 1,558 1.0 ms with a thread per row
+// (a line per lane and load).
+constexpr int EX_WIDE_MIN_D = 64, EX_RW = 8, EX_WARPS = 4;
 template <class P>
-__global__ void __launch_bounds__(128) k_exact_wide(const P *__restrict__ x, int by_point, int64_t n, int32_t d,
-                                                    const int32_t *__restrict__ perm, const int32_t *__restrict__ nsurv,
-                                                    const int32_t *__restrict__ surv, double *__restrict__ rowd2,
-                                                    int32_t *__restrict__ rowj, const int32_t *counters) {
+__global__ void __launch_bounds__(32 * EX_WARPS) k_exact_wide(const P *__restrict__ x, int by_point, int64_t n, int32_t d,
+                                                              const int32_t *__restrict__ perm,
+                                                              const int32_t *__restrict__ nsurv,
+                                                              const int32_t *__restrict__ surv,
+                                                              double *__restrict__ rowd2, int32_t *__restrict__ rowj,
+                                                              const int32_t *counters) {
     if (!mst_active(counters)) return;
-    __shared__ double sq[4][32][33];
+    __shared__ double sq[EX_WARPS][EX_RW][33];
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    const int64_t gs = (int64_t)gridDim.x * 128;
-    for (int64_t r0 = (int64_t)blockIdx.x * 128 + wp * 32; r0 < n; r0 += gs) {
+    const int64_t gs = (int64_t)gridDim.x * EX_WARPS * EX_RW;
+    for (int64_t r0 = ((int64_t)blockIdx.x * EX_WARPS + wp) * EX_RW; r0 < n; r0 += gs) {
         const int64_t r = r0 + lane;
-        const int32_t i = r < n ? perm[r] : -1;
+        const int32_t i = lane < EX_RW && r < n ? perm[r] : -1;
         int c = i >= 0 ? nsurv[r] : 0;
         if (c > TC_SURV) c = 0;
         double best = INFINITY;
@@ -1058,21 +1062,32 @@ __global__ void __launch_bounds__(128) k_exact_wide(const P *__restrict__ x, int
             if (j < 0) jp = -1;
             const int64_t ra = by_point ? (int64_t)i : r, rb = by_point ? (int64_t)j : jp;
             const unsigned live = __ballot_sync(0xffffffffu, jp >= 0);
+            const P *xa[EX_RW], *xb[EX_RW];
+#pragma unroll
+            for (int k = 0; k < EX_RW; ++k) {
+                xa[k] = x + __shfl_sync(0xffffffffu, ra, k) * d;
+                xb[k] = x + __shfl_sync(0xffffffffu, rb, k) * d;
+            }
+            P va[EX_RW], vb[EX_RW];
+            auto load = [&](int t) {
+#pragma unroll
+                for (int k = 0; k < EX_RW; ++k) {
+                    const bool on = (live >> k & 1u) && t < d;
+                    va[k] = on ? xa[k][t] : P(0);
+                    vb[k] = on ? xb[k][t] : P(0);
+                }
+            };
             double e = 0.0;
+            load(lane);
             for (int t0 = 0; t0 < d; t0 += 32) {
-                const int t = t0 + lane;
                 __syncwarp();
-                for (unsigned m = live; m; m &= m - 1u) {
-                    const int k = __ffs(m) - 1;
-                    const int64_t a = __shfl_sync(0xffffffffu, ra, k), b = __shfl_sync(0xffffffffu, rb, k);
-                    double v = 0.0;
-                    if (t < d) {
-                        const double df = __dsub_rn((double)x[a * d + t], (double)x[b * d + t]);
-                        v = __dmul_rn(df, df);
-                    }
-                    sq[wp][k][lane] = v;
+#pragma unroll
+                for (int k = 0; k < EX_RW; ++k) {
+                    const double df = __dsub_rn((double)va[k], (double)vb[k]);
+                    sq[wp][k][lane] = __dmul_rn(df, df);
                 }
                 __syncwarp();
+                load(t0 + 32 + lane);
                 if (jp >= 0) {
                     const int tl = d - t0 < 32 ? d - t0 : 32;
                     for (int u = 0; u < tl; ++u) e = __dadd_rn(e, sq[wp][lane][u]);
@@ -1815,7 +1830,7 @@ cudaError_t tc_sweep_round(TcScratch &T, MstScratch &S, const float *X, int64_t 
                                                    T.nmax_bits, T.nsurv, T.surv, S.counters);
     }
     const bool wide = d >= EX_WIDE_MIN_D;
-    const unsigned wg = (unsigned)(2 * xblocks < xcap ? 2 * xblocks : xcap);
+    const unsigned wg = (unsigned)ceil_div(T.n_pad, EX_RW * EX_WARPS);
 #define ISO_EXACT(PT, XV, BY)                                                                                             \
     (wide ? k_exact_wide<PT><<<wg, 128, 0, ISO_S(s)>>>(XV, BY, T.n_pad, d, T.permp, T.nsurv, T.surv, S.rowd2, S.rowj,      \
                                                        S.counters)                                                        \
@@ -1834,6 +1849,20 @@ cudaError_t tc_sweep_round(TcScratch &T, MstScratch &S, const float *X, int64_t 
     }
 #undef ISO_EXACT
     (void)status;
+    return cudaGetLastError();
+}
+
+cudaError_t tc_key_rows(TcScratch &T, MstScratch &S, const float *X, int64_t n, int32_t d, double mul, double add,
+                        cudaStream_t s) {
+    if (d >= EX_WIDE_MIN_D)
+        k_exact_wide<float><<<(unsigned)ceil_div(n, EX_RW * EX_WARPS), 32 * EX_WARPS, 0, ISO_S(s)>>>(
+            X, 1, n, d, T.permp, T.nsurv, T.surv, S.rowd2, S.rowj, S.counters);
+    else
+        k_exact_tc<float><<<(unsigned)ceil_div(n, 256), 256, 0, ISO_S(s)>>>(X, 1, n, d, T.permp, T.nsurv, T.surv, S.rowd2,
+                                                                          S.rowj, S.counters);
+    k_rescan_tc<float><<<(unsigned)(num_sms() * 4), 256, 0, ISO_S(s)>>>(
+        X, X, n, d, S.comp, S.ovf_rows, T.permp, T.nsurv, nullptr, nullptr, 0, mul, add, 0.0f, T.nmax_bits, S.rowd2, S.rowj,
+        S.counters);
     return cudaGetLastError();
 }
 

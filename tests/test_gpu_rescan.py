@@ -15,7 +15,9 @@ def iso():
         pytest.skip("no CUDA device")
     from paper_1702_04739_gb300 import isoclust
     isoclust.load()
-    return isoclust
+    isoclust.set_sweep_variant(0)                # small sets too take the tensor-core sweep
+    yield isoclust
+    isoclust.set_sweep_variant(-1)
 
 
 def _same_tree(iso, orc, X):
