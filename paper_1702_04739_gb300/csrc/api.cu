@@ -10,6 +10,7 @@
 
 #include "common.cuh"
 #include "mst.cuh"
+#include "sparse.cuh"
 #include "tree.cuh"
 
 namespace iso {
@@ -437,6 +438,14 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     const bool dist = tc_any && !sh && o.precision == ISOCLUST_PREC_AUTO && o.spin_limit == 0 && !TC.stall_test &&
                       tc_forced_variant() < 0 && prune_mode() != 1 && mst_dist_wanted(n, d, dtype);
     float *dmat = nullptr;
+    // rows with few non-zeros, known once the points are looked at: room is
+    // asked for only then
+    bool sp_mst = false;
+    int64_t sp_nnz = 0;
+    SparseRows SP;
+    const bool sp_look = use_tc && !sh && o.precision == ISOCLUST_PREC_AUTO && o.spin_limit == 0 && !TC.stall_test &&
+                         tc_forced_variant() < 0 && prune_mode() != 1 && dtype == ISOCLUST_F32 && d >= SPARSE_MIN_D &&
+                         d <= SPARSE_MAX_D && mst_dist_sparse_wanted(n);
     const int tsplits = tc_any ? tc_splits(n) : 1;
     if (sh) {
         // the sharded work: the tensor-core sweep and the symmetric omega sweep
@@ -482,10 +491,11 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
                            weights64_bytes(n, o.alpha != 0.0) <= SYM_PART_LIMIT;
     auto carve = [&](Arena &A, MstScratch &M, TreeScratch &TS, double **phi, double **om, double **pp, double **omtmp,
                      uint32_t **status) {
-        *status = A.take<uint32_t>(4);
+        *status = A.take<uint32_t>(8);
         M.carve(A, n, splits);
         if (tc_any) TC.carve(A, n, d, tsplits_used, 0, 1, tlists);
-        if (dist) dmat = (float *)A.take<unsigned char>(mst_dist_bytes(n));
+        if (sp_mst) SP.carve(A, n, d, sp_nnz);
+        if (dist || sp_mst) dmat = (float *)A.take<unsigned char>(mst_dist_bytes(n));
         if (weights64) P.sym = (void *)A.take<unsigned char>(weights64_bytes(n, o.alpha != 0.0));
         if (need_labels) {
             TS.carve(A, n);
@@ -527,14 +537,38 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
 
     Events ev;
     ev.rec(0, s);
-    ISO_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t) * 4, s));
+    ISO_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t) * 8, s));
     if (need_labels) ISO_CUDA(cudaMemsetAsync(TS.status, 0, sizeof(uint32_t), s));
     // (status words 2 and 3: the largest magnitude, F64 input)
     ISO_CUDA(check_finite(X, n * (int64_t)d, dtype, status, TC.f64 ? (unsigned long long *)(status + 2) : nullptr, s));
-    struct { uint32_t st, pad; double absmax; } hv = {0, 0, 0.0};
+    // (words 4 to 7: the non-zeros)
+    if (sp_look) ISO_CUDA(sparse_stats((const float *)X, n, d, status + 4, s));
+    struct { uint32_t st, pad; double absmax; unsigned long long nnz; uint32_t longest; float norm_max; } hv = {};
     ISO_CUDA(cudaMemcpyAsync(&hv, status, sizeof(hv), cudaMemcpyDeviceToHost, s));
     ISO_CUDA(cudaStreamSynchronize(s));
     if (hv.st) return map_status(hv.st, false);
+    if (sp_look && sparse_pays(n, d, (int64_t)hv.nnz, hv.norm_max)) {
+        sp_mst = true;
+        sp_nnz = (int64_t)hv.nnz;
+        Arena more;
+        carve(more, M, TS, &phi, &om, &pp, &omtmp, &status);
+        base = scratch_acquire(more.off, s, &st);
+        if (!base) {
+            // no room: as without
+            cudaGetLastError();
+            sp_mst = false;
+            base = scratch_acquire(meas.off, s, &st);
+            if (!base) return st;
+        }
+        A = Arena{(char *)base, (sp_mst ? more.off : meas.off) + 4096, 0, false};
+        carve(A, M, TS, &phi, &om, &pp, &omtmp, &status);
+        if (A.overflow) return fail(ISOCLUST_ERR_INTERNAL, "scratch carve overflow");
+        if (out_phi) phi = out_phi;
+        if (out_omega) om = out_omega;
+        if (out_p) pp = out_p;
+        ISO_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t) * 8, s));
+        if (need_labels) ISO_CUDA(cudaMemsetAsync(TS.status, 0, sizeof(uint32_t), s));
+    }
     ev.rec(1, s);
     bool tc_used = use_tc;
     if (TC.f64 && hv.absmax > TC64_ABS_MIN && hv.absmax < TC64_ABS_MAX) {
@@ -543,8 +577,12 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     }
 
     // Section 2.2 steps 1-2: minimum spanning tree
-    const bool dist_used = dist && tc_used;
-    if (dist_used) {
+    const bool dist_used = sp_mst || (dist && tc_used);
+    if (sp_mst) {
+        tc_clear_last_variant();
+        ISO_CUDA(sparse_build(SP, (const float *)X, s));
+        ISO_CUDA(mst_build_dist(M, TC, dmat, X, n, d, dtype, 0, status, s, &SP, (int32_t)hv.longest));
+    } else if (dist_used) {
         tc_clear_last_variant();
         ISO_CUDA(mst_build_dist(M, TC, dmat, X, n, d, dtype, TC.scale_exp, status, s));
     } else {

@@ -13,6 +13,7 @@
 #include <math.h>
 
 #include "mst.cuh"
+#include "sparse.cuh"
 
 namespace iso {
 namespace {
@@ -107,19 +108,24 @@ __global__ void __launch_bounds__(256) k_dist_tiles(const P *__restrict__ X, int
     }
 }
 
-// One row per block.  INLINE (short rows): a thread keys its own columns, the
-// block's best goes to rowd2 / rowj and to its component's minimum.  Else the
-// columns go to surv for the FP64 keys of long rows, more than SURV of them
-// (exact ties) to the rescan.
+// One row per block.  DK_INLINE (short rows): a thread keys its own columns, the
+// block's best goes to rowd2 / rowj and to its component's minimum.  DK_SPARSE:
+// the same from the rows' non-zeros (a dimension that neither row holds adds
+// nothing to the key); the distances come from a Gram, within err (|x_i|^2 +
+// |x_j|^2) of the true ones.  DK_LIST: the columns go to surv for the FP64 keys
+// of long rows, more than SURV of them (exact ties) to the rescan.
 constexpr int DSC_THREADS = 128, DSC_SURV = 8;
-template <class P, bool INLINE>
+enum : int { DK_INLINE = 0, DK_LIST = 1, DK_SPARSE = 2 };
+template <class P, int KIND>
 __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__ X, int64_t n, int32_t d,
                                                            const float *__restrict__ D, int64_t ld, float mul, float add,
                                                            const int32_t *__restrict__ comp, double *__restrict__ rowd2,
                                                            int32_t *__restrict__ rowj, unsigned long long *__restrict__ cd2,
                                                            int32_t *__restrict__ nsurv, int32_t *__restrict__ surv,
-                                                           int32_t *__restrict__ ovf, int32_t *counters) {
+                                                           int32_t *__restrict__ ovf, int32_t *counters,
+                                                           const SparseRows R, float err) {
     if (!dist_active(counters)) return;
+    constexpr bool INLINE = KIND != DK_LIST;
     __shared__ float smin[DSC_THREADS / 32];
     __shared__ double sb[DSC_THREADS / 32];
     __shared__ int32_t sj[DSC_THREADS / 32];
@@ -128,18 +134,23 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
     const int64_t i = blockIdx.x;
     const int32_t ci = comp[i];
     const float *row = D + i * ld;
+    // the largest and the smallest distance that an entry stands for
+    const float ni = KIND == DK_SPARSE ? R.norm[i].x : 0.0f;
+    auto wide = [&](int64_t j) { return __fmul_ru(err, __fadd_ru(ni, R.norm[j].x)); };
+    auto up = [&](float v, int64_t j) { return KIND == DK_SPARSE ? __fadd_ru(v, wide(j)) : v; };
+    auto down = [&](float v, int64_t j) { return KIND == DK_SPARSE ? __fsub_rd(v, wide(j)) : v; };
     const int64_t n4 = n & ~(int64_t)3;
     if (tid == 0) scnt = 0;
     float m = INFINITY;
     for (int64_t j = 4 * tid; j < n4; j += 4 * DSC_THREADS) {
         const float4 v = *reinterpret_cast<const float4 *>(row + j);
         const int4 c = *reinterpret_cast<const int4 *>(comp + j);
-        if (c.x != ci) m = fminf(m, v.x);
-        if (c.y != ci) m = fminf(m, v.y);
-        if (c.z != ci) m = fminf(m, v.z);
-        if (c.w != ci) m = fminf(m, v.w);
+        if (c.x != ci) m = fminf(m, up(v.x, j));
+        if (c.y != ci) m = fminf(m, up(v.y, j + 1));
+        if (c.z != ci) m = fminf(m, up(v.z, j + 2));
+        if (c.w != ci) m = fminf(m, up(v.w, j + 3));
     }
-    if (n4 + tid < n && comp[n4 + tid] != ci) m = fminf(m, row[n4 + tid]);
+    if (n4 + tid < n && comp[n4 + tid] != ci) m = fminf(m, up(row[n4 + tid], n4 + tid));
     for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) smin[wp] = m;
     __syncthreads();
@@ -151,9 +162,21 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
     auto see = [&](int64_t j) {
         if constexpr (INLINE) {
             double e = 0.0;
-            for (int t = 0; t < d; ++t) {
-                const double df = __dsub_rn((double)X[i * d + t], (double)X[j * d + t]);
-                e = __dadd_rn(e, __dmul_rn(df, df));
+            if constexpr (KIND == DK_SPARSE) {
+                int32_t a = R.rowptr[i], b = R.rowptr[j];
+                const int32_t a1 = R.rowptr[i + 1], b1 = R.rowptr[j + 1];
+                while (a < a1 || b < b1) {
+                    const int32_t ta = a < a1 ? R.rcol[a] : INT32_MAX, tb = b < b1 ? R.rcol[b] : INT32_MAX;
+                    double df = 0.0;
+                    if (ta <= tb) df = (double)R.rval[a++];
+                    if (tb <= ta) df = __dsub_rn(df, (double)R.rval[b++]);
+                    e = __dadd_rn(e, __dmul_rn(df, df));
+                }
+            } else {
+                for (int t = 0; t < d; ++t) {
+                    const double df = __dsub_rn((double)X[i * d + t], (double)X[j * d + t]);
+                    e = __dadd_rn(e, __dmul_rn(df, df));
+                }
             }
             if (bestj < 0 || key_less(e, (int32_t)i, (int32_t)j, best, (int32_t)i, bestj)) {
                 best = e;
@@ -166,14 +189,14 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
     };
     for (int64_t j = 4 * tid; j < n4; j += 4 * DSC_THREADS) {
         const float4 v = *reinterpret_cast<const float4 *>(row + j);
-        if (fminf(fminf(v.x, v.y), fminf(v.z, v.w)) > thr) continue;
+        if (KIND != DK_SPARSE && fminf(fminf(v.x, v.y), fminf(v.z, v.w)) > thr) continue;
         const int4 c = *reinterpret_cast<const int4 *>(comp + j);
-        if (c.x != ci && v.x <= thr) see(j);
-        if (c.y != ci && v.y <= thr) see(j + 1);
-        if (c.z != ci && v.z <= thr) see(j + 2);
-        if (c.w != ci && v.w <= thr) see(j + 3);
+        if (c.x != ci && down(v.x, j) <= thr) see(j);
+        if (c.y != ci && down(v.y, j + 1) <= thr) see(j + 1);
+        if (c.z != ci && down(v.z, j + 2) <= thr) see(j + 2);
+        if (c.w != ci && down(v.w, j + 3) <= thr) see(j + 3);
     }
-    if (n4 + tid < n && comp[n4 + tid] != ci && row[n4 + tid] <= thr) see(n4 + tid);
+    if (n4 + tid < n && comp[n4 + tid] != ci && down(row[n4 + tid], n4 + tid) <= thr) see(n4 + tid);
     if constexpr (INLINE) {
         auto take = [&](double e, int32_t j) {
             if (j >= 0 && (bestj < 0 || key_less(e, (int32_t)i, j, best, (int32_t)i, bestj))) {
@@ -342,45 +365,57 @@ constexpr int64_t MST_DIST_MAX_F64 = 100000000;        // n^2 d
 // kernels of their own .22; 4,900 .88, .59)
 constexpr int32_t MST_DIST_INLINE_MAX_D = 32;
 
+// Rows by their non-zeros: while the matrix stays within 16 GiB.
+bool mst_dist_sparse_wanted(int64_t n) { return n <= 65536; }
+
 bool mst_dist_wanted(int64_t n, int32_t d, int dtype) {
     if (n < 2 || n > MST_DIST_MAX_N) return false;
     return dtype == ISOCLUST_F32 || (d <= 2 * MST_DIST_INLINE_MAX_D && n * n <= MST_DIST_MAX_F64 / d);
 }
 
 cudaError_t mst_build_dist(MstScratch &S, TcScratch &T, float *D, const void *X, int64_t n, int32_t d, int dtype,
-                           int scale_exp, uint32_t *status, cudaStream_t s) {
+                           int scale_exp, uint32_t *status, cudaStream_t s, const SparseRows *sp, int32_t longest) {
     const int64_t Tn = ceil_div(n, DS_T), ld = Tn * DS_T;
     const unsigned tiles = (unsigned)(Tn * (Tn + 1) / 2);
-    const bool f64 = dtype == ISOCLUST_F64, inl = f64 || d <= MST_DIST_INLINE_MAX_D;
+    const bool f64 = dtype == ISOCLUST_F64, inl = sp || f64 || d <= MST_DIST_INLINE_MAX_D;
     const double sc = f64 ? ldexp(1.0, -scale_exp) : 1.0;
     cudaError_t e;
     k_dist_init<<<(unsigned)ceil_div(n < 8 ? 8 : n, TPB), TPB, 0, ISO_S(s)>>>(S.comp, S.cd2, S.cpair, inl ? nullptr : T.permp, n,
                                                                             S.counters);
-    if (f64)
+    if (sp) {
+        if ((e = sparse_dist(*sp, D, ld, s))) return e;
+    } else if (f64)
         k_dist_tiles<double><<<tiles, 256, 0, ISO_S(s)>>>((const double *)X, n, d, sc, Tn, D, ld);
     else
         k_dist_tiles<float><<<tiles, 256, 0, ISO_S(s)>>>((const float *)X, n, d, sc, Tn, D, ld);
     // any column within m (1 + e) / (1 - e) + 2 add of the row's FP32 minimum
     // can hold the exact best (e: 10 % above the bound of the distances)
-    const double er = 1.1 * (double)(d + 3) * 5.9604644775390625e-08;
-    const double mul = (1.0 + er) / (1.0 - er), add = (double)(d + 1) * 1.401298464324817e-45 * 4.0;
+    const double u = 5.9604644775390625e-08, er = 1.1 * (double)(d + 3) * u;
+    const double mul = sp ? 1.0 : (1.0 + er) / (1.0 - er), add = (double)(d + 1) * 1.401298464324817e-45 * 4.0;
     const float mul32 = (float)(mul * (1.0 + 1e-6)), add32 = (float)(2.01 * add) + 1.401298464324817e-45f;
+    // A Gram's distance: the products' sums (a rounding per entry of the shorter
+    // row, 2^-24 of |x_i| |x_j| <= (|x_i|^2 + |x_j|^2) / 2 each, twice), the norms
+    // and the two last operations: within (longest + 5) 2^-24 (|x_i|^2 + |x_j|^2)
+    const float err = sp ? (float)(1.1 * (double)(longest + 6) * u) : 0.0f;
+    const SparseRows none, &R0 = sp ? *sp : none;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if ((e = cudaStreamIsCapturing(s, &cs))) return e;
     const bool ask = cs == cudaStreamCaptureStatusNone;
     int R = 1;                                         // components at least halve per round
     while ((int64_t(1) << (R - 1)) < n) ++R;
     for (int r = 0; r < R; ++r) {
-#define ISO_SCAN(PT, INL)                                                                                              \
-    k_dist_scan<PT, INL><<<(unsigned)n, DSC_THREADS, 0, ISO_S(s)>>>((const PT *)X, n, d, D, ld, mul32, add32, S.comp,   \
+#define ISO_SCAN(PT, KIND)                                                                                             \
+    k_dist_scan<PT, KIND><<<(unsigned)n, DSC_THREADS, 0, ISO_S(s)>>>((const PT *)X, n, d, D, ld, mul32, add32, S.comp,   \
                                                                     S.rowd2, S.rowj, S.cd2, T.nsurv, T.surv,           \
-                                                                    S.ovf_rows, S.counters)
-        if (f64) {
-            ISO_SCAN(double, true);
+                                                                    S.ovf_rows, S.counters, R0, err)
+        if (sp) {
+            ISO_SCAN(float, DK_SPARSE);
+        } else if (f64) {
+            ISO_SCAN(double, DK_INLINE);
         } else if (inl) {
-            ISO_SCAN(float, true);
+            ISO_SCAN(float, DK_INLINE);
         } else {
-            ISO_SCAN(float, false);
+            ISO_SCAN(float, DK_LIST);
             if ((e = tc_key_rows(T, S, (const float *)X, n, d, mul, add, s))) return e;
             if ((e = mst_component_minima(S, n, s))) return e;
         }
