@@ -22,7 +22,8 @@ cudaError_t weights_launch_sym(const float *X, int64_t n, int32_t d, double sigm
                                const unsigned long long *nnbits, double *omega, void *part,
                                unsigned long long *tile_counts, const uint8_t *need, cudaEvent_t *kev,
                                cudaStream_t s, const Shard *sh = nullptr, double *part64 = nullptr,
-                               void *gram = nullptr, uint32_t *status = nullptr, uint64_t wait_cycles = 0);
+                               void *gram = nullptr, uint32_t *status = nullptr, uint64_t wait_cycles = 0,
+                               const SparseRows *sp = nullptr);
 float omega_zskip(int64_t n);
 size_t weights64_bytes(int64_t n, bool with_p);
 cudaError_t weights64_launch(const void *X, int64_t n, int32_t d, int dtype, double sigma, double alpha,
@@ -517,7 +518,7 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
             if (symmetric) P.sym = (void *)A.take<unsigned char>(weights_sym_bytes(n, d));
             if (symmetric && use_tc) P.need = A.take<uint8_t>((size_t)ceil_div(n, 64) * ceil_div(n, 64));
             if (sh) P.part64 = A.take<double>(n);
-            if (gram) P.gram = (void *)A.take<unsigned char>(omega_tc_bytes(n, d, tri_items(n)), 1024);
+            if (gram) P.gram = (void *)A.take<unsigned char>(omega_tc_bytes(n, sp_mst ? 0 : d, tri_items(n)), 1024);
         }
     };
     MstScratch M;
@@ -634,14 +635,19 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
                 ISO_CUDA(cudaMemsetAsync(P.tiles, 0, 4 * sizeof(unsigned long long), s));
                 if (symmetric) {
                     // the tensor cores decide which pairs of 64-row tiles can hold a term
-                    if (use_tc) {
+                    const bool lists = sp_mst && gram;
+                    if (lists) {
+                        // the lists again, in omega's row order
+                        ISO_CUDA(sparse_build(SP, P.Xp, s));
+                    } else if (use_tc) {
                         ISO_CUDA(tc_omega_screen(TC, P.Xp, n, d, P.nnp, sigma, (double)omega_zskip(n), P.need,
                                                  ceil_div(n, 64), s));
                         k_or_err_api<<<1, 1, 0, ISO_S(s)>>>(TC.err, status);
                     }
                     ISO_CUDA(weights_launch_sym(P.Xp, n, d, sigma, o.include_self, P.nnp, P.omp, P.sym, P.tiles,
                                                 use_tc ? P.need : nullptr, ev.ok ? ev.e + 8 : nullptr, s, sh,
-                                                P.part64, gram ? P.gram : nullptr, status, o.spin_limit));
+                                                P.part64, gram ? P.gram : nullptr, status, o.spin_limit,
+                                                lists ? &SP : nullptr));
                 }
                 else
                     ISO_CUDA(weights_launch(P.Xp, n, d, dtype, false, sigma, o.alpha, o.include_self, P.nnp, P.omp,

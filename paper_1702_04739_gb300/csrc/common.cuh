@@ -107,11 +107,12 @@ size_t omega_tc_bytes(int64_t rows, int32_t d, int64_t nitems);
 // The kept tile pairs' terms (tskip 0) with the Gram on the tensor cores:
 // row and column partials and flags as k_weights_sym writes them.
 // kev (may be null): two events recorded around the kernel.
+struct SparseRows;
 cudaError_t omega_tc_launch(void *scratch, size_t scratch_bytes, const OmegaItems &L, const float *Xp, int64_t rows,
                             int32_t d, const float *cen, const float2 *shdw, const uint8_t *tskip, float is_h, float is_l,
                             float zskip, const ExpTable &tab, uint8_t *flags, float2 *rpart, float2 *cpart,
                             unsigned long long *tile_counts, int shard_rank, int shard_world, uint32_t *err,
-                            uint64_t wait_cycles, cudaStream_t s, cudaEvent_t *kev);
+                            uint64_t wait_cycles, cudaStream_t s, cudaEvent_t *kev, const SparseRows *sp = nullptr);
 
 // ---------------------------------------------------------------- helpers
 __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }

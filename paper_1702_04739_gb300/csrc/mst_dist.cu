@@ -114,9 +114,11 @@ __global__ void __launch_bounds__(256) k_dist_tiles(const P *__restrict__ X, int
 // nothing to the key); the distances come from a Gram, within err (|x_i|^2 +
 // |x_j|^2) of the true ones.  DK_LIST: the columns go to surv for the FP64 keys
 // of long rows, more than SURV of them (exact ties) to the rescan.
-constexpr int DSC_THREADS = 128, DSC_SURV = 8;
+// A thread whose own columns hold none within the margin does not look again:
+// of long rows (512 threads) the second look reads a tenth of the matrix.
+constexpr int DSC_SURV = 8;
 enum : int { DK_INLINE = 0, DK_LIST = 1, DK_SPARSE = 2 };
-template <class P, int KIND>
+template <class P, int KIND, int DSC_THREADS>
 __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__ X, int64_t n, int32_t d,
                                                            const float *__restrict__ D, int64_t ld, float mul, float add,
                                                            const int32_t *__restrict__ comp, double *__restrict__ rowd2,
@@ -141,16 +143,20 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
     auto down = [&](float v, int64_t j) { return KIND == DK_SPARSE ? __fsub_rd(v, wide(j)) : v; };
     const int64_t n4 = n & ~(int64_t)3;
     if (tid == 0) scnt = 0;
-    float m = INFINITY;
+    float m = INFINITY, low = INFINITY;
+    auto first = [&](float v, int64_t j) {
+        m = fminf(m, up(v, j));
+        low = fminf(low, down(v, j));
+    };
     for (int64_t j = 4 * tid; j < n4; j += 4 * DSC_THREADS) {
         const float4 v = *reinterpret_cast<const float4 *>(row + j);
         const int4 c = *reinterpret_cast<const int4 *>(comp + j);
-        if (c.x != ci) m = fminf(m, up(v.x, j));
-        if (c.y != ci) m = fminf(m, up(v.y, j + 1));
-        if (c.z != ci) m = fminf(m, up(v.z, j + 2));
-        if (c.w != ci) m = fminf(m, up(v.w, j + 3));
+        if (c.x != ci) first(v.x, j);
+        if (c.y != ci) first(v.y, j + 1);
+        if (c.z != ci) first(v.z, j + 2);
+        if (c.w != ci) first(v.w, j + 3);
     }
-    if (n4 + tid < n && comp[n4 + tid] != ci) m = fminf(m, up(row[n4 + tid], n4 + tid));
+    if (n4 + tid < n && comp[n4 + tid] != ci) first(row[n4 + tid], n4 + tid);
     for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) smin[wp] = m;
     __syncthreads();
@@ -187,15 +193,16 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
             if (q < DSC_SURV) surv[i * DSC_SURV + q] = (int32_t)j;
         }
     };
-    for (int64_t j = 4 * tid; j < n4; j += 4 * DSC_THREADS) {
-        const float4 v = *reinterpret_cast<const float4 *>(row + j);
-        if (KIND != DK_SPARSE && fminf(fminf(v.x, v.y), fminf(v.z, v.w)) > thr) continue;
-        const int4 c = *reinterpret_cast<const int4 *>(comp + j);
-        if (c.x != ci && down(v.x, j) <= thr) see(j);
-        if (c.y != ci && down(v.y, j + 1) <= thr) see(j + 1);
-        if (c.z != ci && down(v.z, j + 2) <= thr) see(j + 2);
-        if (c.w != ci && down(v.w, j + 3) <= thr) see(j + 3);
-    }
+    if (low <= thr)
+        for (int64_t j = 4 * tid; j < n4; j += 4 * DSC_THREADS) {
+            const float4 v = *reinterpret_cast<const float4 *>(row + j);
+            if (KIND != DK_SPARSE && fminf(fminf(v.x, v.y), fminf(v.z, v.w)) > thr) continue;
+            const int4 c = *reinterpret_cast<const int4 *>(comp + j);
+            if (c.x != ci && down(v.x, j) <= thr) see(j);
+            if (c.y != ci && down(v.y, j + 1) <= thr) see(j + 1);
+            if (c.z != ci && down(v.z, j + 2) <= thr) see(j + 2);
+            if (c.w != ci && down(v.w, j + 3) <= thr) see(j + 3);
+        }
     if (n4 + tid < n && comp[n4 + tid] != ci && down(row[n4 + tid], n4 + tid) <= thr) see(n4 + tid);
     if constexpr (INLINE) {
         auto take = [&](double e, int32_t j) {
@@ -404,18 +411,19 @@ cudaError_t mst_build_dist(MstScratch &S, TcScratch &T, float *D, const void *X,
     int R = 1;                                         // components at least halve per round
     while ((int64_t(1) << (R - 1)) < n) ++R;
     for (int r = 0; r < R; ++r) {
-#define ISO_SCAN(PT, KIND)                                                                                             \
-    k_dist_scan<PT, KIND><<<(unsigned)n, DSC_THREADS, 0, ISO_S(s)>>>((const PT *)X, n, d, D, ld, mul32, add32, S.comp,   \
+#define ISO_SCAN(PT, KIND, NT)                                                                                            \
+    k_dist_scan<PT, KIND, NT><<<(unsigned)n, NT, 0, ISO_S(s)>>>((const PT *)X, n, d, D, ld, mul32, add32, S.comp,   \
                                                                     S.rowd2, S.rowj, S.cd2, T.nsurv, T.surv,           \
                                                                     S.ovf_rows, S.counters, R0, err)
         if (sp) {
-            ISO_SCAN(float, DK_SPARSE);
+            if (n > MST_DIST_MAX_N) ISO_SCAN(float, DK_SPARSE, 512);
+            else ISO_SCAN(float, DK_SPARSE, 128);
         } else if (f64) {
-            ISO_SCAN(double, DK_INLINE);
+            ISO_SCAN(double, DK_INLINE, 128);
         } else if (inl) {
-            ISO_SCAN(float, DK_INLINE);
+            ISO_SCAN(float, DK_INLINE, 128);
         } else {
-            ISO_SCAN(float, DK_LIST);
+            ISO_SCAN(float, DK_LIST, 128);
             if ((e = tc_key_rows(T, S, (const float *)X, n, d, mul, add, s))) return e;
             if ((e = mst_component_minima(S, n, s))) return e;
         }

@@ -881,7 +881,7 @@ cudaError_t weights_launch_sym(const float *X, int64_t n, int32_t d, double sigm
                                const unsigned long long *nnbits, double *omega, void *part,
                                unsigned long long *tile_counts, const uint8_t *need, cudaEvent_t *kev,
                                cudaStream_t s, const Shard *sh, double *part64, void *gram, uint32_t *status,
-                               uint64_t wait_cycles) {
+                               uint64_t wait_cycles, const SparseRows *sp) {
     static const ExpTable tab = make_exp_table();
     const double is = 1.0 / sigma;
     const float is_h = (float)is;
@@ -894,20 +894,26 @@ cudaError_t weights_launch_sym(const float *X, int64_t n, int32_t d, double sigm
     const SymParts P = sym_parts(part, items, n, T, d);
     const unsigned grid = (unsigned)(num_sms() * 2);
     k_shift_dw<<<(unsigned)ceil_div(n, 256), 256, 0, ISO_S(s)>>>(nnbits, n, is, P.shdw);
-    k_tile_bounds<<<(unsigned)T, 64, 0, ISO_S(s)>>>(X, n, d, P.shdw, nullptr, P.cen, P.rad, P.msh);
-    k_tile_pair_skip<false><<<(unsigned)(num_sms() * 8), 256, 0, ISO_S(s)>>>(P.cen, P.rad, P.msh, d, T, items, nullptr,
-                                                                            is_h, zskip, shrink, need, P.tskip);
     cudaError_t err;
+    if (sp) {
+        // rows as lists: no pair of tiles is left out ahead (a term costs less than
+        // the bounds that would spare it)
+        if ((err = cudaMemsetAsync(P.tskip, 0, (size_t)items, s))) return err;
+    } else {
+        k_tile_bounds<<<(unsigned)T, 64, 0, ISO_S(s)>>>(X, n, d, P.shdw, nullptr, P.cen, P.rad, P.msh);
+        k_tile_pair_skip<false><<<(unsigned)(num_sms() * 8), 256, 0, ISO_S(s)>>>(P.cen, P.rad, P.msh, d, T, items, nullptr,
+                                                                                is_h, zskip, shrink, need, P.tskip);
+    }
     // sharded: the items of other ranks hold nothing here
     if (sh && (err = cudaMemsetAsync(P.flags, 0, (size_t)items, s))) return err;
-    if (gram && need) {
+    if (gram && (need || sp)) {
         OmegaItems L;
         L.nitems = items;
         L.T = T;
         L.n = n;
-        if ((err = omega_tc_launch(gram, omega_tc_bytes(n, d, items), L, X, n, d, P.cen, P.shdw, P.tskip, is_h, is_l, zskip,
+        if ((err = omega_tc_launch(gram, omega_tc_bytes(n, sp ? 0 : d, items), L, X, n, d, P.cen, P.shdw, P.tskip, is_h, is_l, zskip,
                                    tab, P.flags, P.rpart, P.cpart, tile_counts, sh ? sh->rank : 0, sh ? sh->world : 1,
-                                   status, wait_cycles, s, kev)))
+                                   status, wait_cycles, s, kev, sp)))
             return err;
     } else {
         if (kev) record_event(kev[0], s);

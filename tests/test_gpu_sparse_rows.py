@@ -67,3 +67,24 @@ def test_density_rule(iso, share, sparse):
     X[:, : d // 16 + (0 if sparse else 1)] = np.random.default_rng(1).normal(size=(n, d // 16 + (0 if sparse else 1)))
     iso.cluster_mst(torch.from_numpy(X).cuda())
     assert (iso.last_profile()["mst_tiles_full"] == 0) == sparse
+
+
+def _bound(orc, X, sigma):
+    # d2 to 2^-46 (of its parts where they do not cancel to under a quarter of them), so y = d /
+    # sigma to half of that relatively, every term to y times it; 4: the exponential and the sums
+    nn, nd2 = orc.nn_rows(X, np.arange(X.shape[0]))
+    return 2.0 ** -45 * max(1.0, math.sqrt(X.shape[1] / 64.0)) * (np.sqrt(nd2) / sigma + 4.0)
+
+
+@pytest.mark.parametrize("n,d", SHAPES[:-1] + [(2500, 512)])
+@pytest.mark.parametrize("kind", ["plain", "odd", "shared"])
+def test_omega(iso, oracle_lib, n, d, kind):
+    X = _rows(n, d, kind)
+    Xd = torch.from_numpy(X).cuda()
+    for sigma in (1.0, 0.3):
+        ref, _ = oracle_lib.weights(X, sigma)
+        iso.set_omega_gram(1)
+        om = iso.cluster_detail(Xd, 1, sigma)["omega"].cpu().numpy()
+        assert iso.last_profile()["omega_symmetric"] == 3
+        iso.set_omega_gram(-1)
+        assert (np.abs(om - ref) <= _bound(oracle_lib, X, sigma) * ref).all()
