@@ -14,9 +14,10 @@
 #include "tree.cuh"
 
 namespace iso {
+size_t weights_dw_bytes(int64_t n);
 cudaError_t weights_launch(const void *X, int64_t n, int32_t d, int dtype, bool fp64_path, double sigma,
                            double alpha, int include_self, const unsigned long long *nnbits, double *omega,
-                           double *p, unsigned long long *tile_counts, cudaStream_t s);
+                           double *p, unsigned long long *tile_counts, cudaStream_t s, void *part = nullptr);
 size_t weights_sym_bytes(int64_t n, int32_t d);
 cudaError_t weights_launch_sym(const float *X, int64_t n, int32_t d, double sigma, int include_self,
                                const unsigned long long *nnbits, double *omega, void *part,
@@ -516,6 +517,7 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
             P.omp = A.take<double>(n);
             P.pp = A.take<double>(n);
             if (symmetric) P.sym = (void *)A.take<unsigned char>(weights_sym_bytes(n, d));
+            else if (o.alpha != 0.0) P.sym = (void *)A.take<unsigned char>(weights_dw_bytes(n));
             if (symmetric && use_tc) P.need = A.take<uint8_t>((size_t)ceil_div(n, 64) * ceil_div(n, 64));
             if (sh) P.part64 = A.take<double>(n);
             if (gram) P.gram = (void *)A.take<unsigned char>(omega_tc_bytes(n, sp_mst ? 0 : d, tri_items(n)), 1024);
@@ -651,7 +653,7 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
                 }
                 else
                     ISO_CUDA(weights_launch(P.Xp, n, d, dtype, false, sigma, o.alpha, o.include_self, P.nnp, P.omp,
-                                            P.pp, P.tiles, s));
+                                            P.pp, P.tiles, s, P.sym));
                 k_scatter_rows<<<gb, TPB, 0, ISO_S(s)>>>(P.omp, P.perm, n, om_out);
                 if (symmetric)
                     ISO_CUDA(cudaMemsetAsync(pp, 0, sizeof(double) * n, s));

@@ -52,12 +52,16 @@ struct RowAcc {
 // plain FP32; if no pair can have a term above e^-zskip of its row's
 // largest term (a rigorous lower bound on z from the FP32 error bound), the
 // tile pair is skipped.  Skipped terms total < n e^-zskip relative.
+// Split (part != nullptr): blockIdx.y takes its share of the column tiles and
+// leaves the rows' sums in part [split][n] for k_weights_dw_merge.  A block per
+// 64 rows leaves half the SMs without work below 10,000 rows: 4,898 x 11 with
+// potentials 0.72 ms by 77 blocks.
 template <bool WITH_P, bool SCREEN>
 __global__ void __launch_bounds__(TPB, 2)
 k_weights_dw(const float *__restrict__ X, int64_t n, int32_t d, const unsigned long long *__restrict__ nnbits,
              float is_h, float is_l, double inv_sigma, ExpTable tabv, double alpha, int include_self,
              float zskip, float scr_shrink, double *__restrict__ omega, double *__restrict__ pout,
-             unsigned long long *__restrict__ tile_counts) {
+             unsigned long long *__restrict__ tile_counts, float4 *__restrict__ part) {
     __shared__ __align__(16) float As[WDC][WPAD];
     __shared__ __align__(16) float Bs[WDC][WPAD];
     __shared__ float2 tab[64];
@@ -86,8 +90,9 @@ k_weights_dw(const float *__restrict__ X, int64_t n, int32_t d, const unsigned l
     for (int i = 0; i < 4; ++i) acc[i] = RowAcc{0.f, 0.f, 0.f, 0.f};
 
     const int64_t ntiles = ceil_div(n, WT);
+    const int64_t ct0 = ntiles * blockIdx.y / gridDim.y, ct1 = ntiles * (blockIdx.y + 1) / gridDim.y;
     unsigned long long dw_tiles = 0;
-    for (int64_t ct = 0; ct < ntiles; ++ct) {
+    for (int64_t ct = ct0; ct < ct1; ++ct) {
         const int64_t col0 = ct * WT;
         if (SCREEN) {
             float A32[4][4];
@@ -210,7 +215,7 @@ k_weights_dw(const float *__restrict__ X, int64_t n, int32_t d, const unsigned l
         }
     }
     if (SCREEN && tid == 0) {
-        atomicAdd(tile_counts + 0, (unsigned long long)ntiles);
+        atomicAdd(tile_counts + 0, (unsigned long long)(ct1 - ct0));
         atomicAdd(tile_counts + 1, dw_tiles);
     }
     // merge the 16 column-threads of each row in fixed order
@@ -233,6 +238,10 @@ k_weights_dw(const float *__restrict__ X, int64_t n, int32_t d, const unsigned l
                 dw_add(h, l, mw[tid][s][0], mw[tid][s][1]);
                 if (WITH_P) dw_add(qh, ql, mp[tid][s][0], mp[tid][s][1]);
             }
+            if (part) {
+                part[(int64_t)blockIdx.y * n + r] = make_float4(h, l, qh, ql);
+                return;
+            }
             // the shift actually applied to this row's terms was the
             // double-word (fh, fl) of sh; fh + fl is exact in FP64
             double nd2 = bitsd(nnbits[r]);
@@ -246,6 +255,27 @@ k_weights_dw(const float *__restrict__ X, int64_t n, int32_t d, const unsigned l
             if (WITH_P && pout) pout[r] = __dmul_rn(alpha, __dadd_rn((double)qh, (double)ql));
         }
     }
+}
+
+// the splits' sums of a row, in order, and its weight as in k_weights_dw
+__global__ void k_weights_dw_merge(const float4 *__restrict__ part, int splits, int64_t n,
+                                   const unsigned long long *__restrict__ nnbits, double inv_sigma, double alpha,
+                                   int include_self, double *__restrict__ omega, double *__restrict__ pout) {
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= n) return;
+    float h = 0.f, l = 0.f, qh = 0.f, ql = 0.f;
+    for (int q = 0; q < splits; ++q) {
+        const float4 v = part[(int64_t)q * n + r];
+        dw_add(h, l, v.x, v.y);
+        dw_add(qh, ql, v.z, v.w);
+    }
+    const double nd2 = bitsd(nnbits[r]);
+    const double sh = isfinite(nd2) ? __dmul_rn(__dsqrt_rn(nd2), inv_sigma) : 0.0;
+    const float fh = (float)sh, fl = (float)(sh - (double)fh);
+    double w = __dmul_rn(exp(-__dadd_rn((double)fh, (double)fl)), __dadd_rn((double)h, (double)l));
+    if (include_self) w = __dadd_rn(w, 1.0);
+    omega[r] = w;
+    pout[r] = __dmul_rn(alpha, __dadd_rn((double)qh, (double)ql));
 }
 
 // exp(-(d / sigma - shift)) for a double-word distance (r, dl); false when
@@ -991,9 +1021,20 @@ cudaError_t weights_launch_sym_sets(const float *Xp, int64_t n_pad, int32_t d, d
     return cudaGetLastError();
 }
 
+// Column splits of k_weights_dw: four waves of two blocks per SM, at least
+// four column tiles each.
+static int weights_dw_splits(int64_t n) {
+    const int64_t g = ceil_div(n, WT);
+    int64_t ns = ceil_div((int64_t)num_sms() * 8, g);
+    if (ns > g / 4) ns = g / 4;
+    return (int)(ns < 1 ? 1 : (ns > 16 ? 16 : ns));
+}
+
+size_t weights_dw_bytes(int64_t n) { return (size_t)weights_dw_splits(n) * (size_t)n * sizeof(float4); }
+
 cudaError_t weights_launch(const void *X, int64_t n, int32_t d, int dtype, bool fp64_path, double sigma,
                            double alpha, int include_self, const unsigned long long *nnbits, double *omega,
-                           double *p, unsigned long long *tile_counts, cudaStream_t s) {
+                           double *p, unsigned long long *tile_counts, cudaStream_t s, void *part) {
     if (fp64_path || dtype == ISOCLUST_F64) {
         unsigned g = (unsigned)ceil_div(n, TPB);
         if (dtype == ISOCLUST_F64)
@@ -1016,15 +1057,23 @@ cudaError_t weights_launch(const void *X, int64_t n, int32_t d, int dtype, bool 
     unsigned g = (unsigned)ceil_div(n, WT);
     const bool with_p = alpha != 0.0 && p;
     const bool screen = !with_p && tile_counts != nullptr;
-    if (with_p)
+    const int ns = with_p && part ? weights_dw_splits(n) : 1;
+    if (ns > 1) {
+        k_weights_dw<true, false><<<dim3(g, (unsigned)ns), TPB, 0, ISO_S(s)>>>(
+            (const float *)X, n, d, nnbits, is_h, is_l, is, tab, alpha, include_self, zskip, shrink, omega, p, tile_counts,
+            (float4 *)part);
+        k_weights_dw_merge<<<(unsigned)ceil_div(n, 128), 128, 0, ISO_S(s)>>>((const float4 *)part, ns, n, nnbits, is, alpha,
+                                                                            include_self, omega, p);
+    } else if (with_p)
         k_weights_dw<true, false><<<g, TPB, 0, ISO_S(s)>>>((const float *)X, n, d, nnbits, is_h, is_l, is, tab, alpha,
-                                                          include_self, zskip, shrink, omega, p, tile_counts);
+                                                          include_self, zskip, shrink, omega, p, tile_counts, nullptr);
     else if (screen)
         k_weights_dw<false, true><<<g, TPB, 0, ISO_S(s)>>>((const float *)X, n, d, nnbits, is_h, is_l, is, tab, alpha,
-                                                          include_self, zskip, shrink, omega, p, tile_counts);
+                                                          include_self, zskip, shrink, omega, p, tile_counts, nullptr);
     else
         k_weights_dw<false, false><<<g, TPB, 0, ISO_S(s)>>>((const float *)X, n, d, nnbits, is_h, is_l, is, tab,
-                                                           alpha, include_self, zskip, shrink, omega, p, tile_counts);
+                                                           alpha, include_self, zskip, shrink, omega, p, tile_counts,
+                                                           nullptr);
     if (!with_p && p) {
         cudaError_t e2 = cudaMemsetAsync(p, 0, sizeof(double) * n, s);
         if (e2 != cudaSuccess) return e2;
