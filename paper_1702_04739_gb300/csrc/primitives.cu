@@ -129,10 +129,9 @@ __global__ void merge_pass(const uint64_t *__restrict__ kin, const int32_t *__re
 // SORT_CHUNK elements with the same stable rank merge, run widths 1 to
 // SORT_CHUNK / 2, then the global passes continue from SORT_CHUNK.
 constexpr int SORT_CHUNK = 2048, SORT_THREADS = 1024;
-__global__ void __launch_bounds__(SORT_THREADS) chunk_sort(const uint64_t *__restrict__ kin,
-                                                           const int32_t *__restrict__ vin,
-                                                           uint64_t *__restrict__ kout, int32_t *__restrict__ vout,
-                                                           int64_t n) {
+// (in and out may be the same arrays: a block reads its chunk before it writes it)
+__global__ void __launch_bounds__(SORT_THREADS) chunk_sort(const uint64_t *kin, const int32_t *vin, uint64_t *kout,
+                                                           int32_t *vout, int64_t n) {
     __shared__ uint64_t sk[2][SORT_CHUNK];
     __shared__ int32_t sv[2][SORT_CHUNK];
     const int64_t base = (int64_t)blockIdx.x * SORT_CHUNK;
@@ -182,8 +181,13 @@ cudaError_t sort_pairs_u64(uint64_t *keys, int32_t *vals, uint64_t *kbuf, int32_
     if (n <= 1) return cudaSuccess;
     uint64_t *ka = keys, *kb = kbuf;
     int32_t *va = vals, *vb = vbuf;
-    chunk_sort<<<(unsigned)ceil_div(n, SORT_CHUNK), SORT_THREADS, 0, ISO_S(s)>>>(ka, va, kb, vb, n);
-    {
+    // the chunks go where an even number of merge passes leaves the result in keys
+    int passes = 0;
+    for (int64_t w = SORT_CHUNK; w < n; w <<= 1) ++passes;
+    const bool in_place = passes % 2 == 0;
+    chunk_sort<<<(unsigned)ceil_div(n, SORT_CHUNK), SORT_THREADS, 0, ISO_S(s)>>>(ka, va, in_place ? ka : kb,
+                                                                                in_place ? va : vb, n);
+    if (!in_place) {
         uint64_t *tk = ka; ka = kb; kb = tk;
         int32_t *tv = va; va = vb; vb = tv;
     }
@@ -191,12 +195,6 @@ cudaError_t sort_pairs_u64(uint64_t *keys, int32_t *vals, uint64_t *kbuf, int32_
         merge_pass<<<(unsigned)ceil_div(n, 256), 256, 0, ISO_S(s)>>>(ka, va, kb, vb, n, w);
         uint64_t *tk = ka; ka = kb; kb = tk;
         int32_t *tv = va; va = vb; vb = tv;
-    }
-    if (ka != keys) {
-        cudaError_t e = cudaMemcpyAsync(keys, ka, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess) return e;
-        e = cudaMemcpyAsync(vals, va, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
 }

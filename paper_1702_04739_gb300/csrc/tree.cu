@@ -192,6 +192,146 @@ __global__ void k_wyllie(const int32_t *__restrict__ sin, const int32_t *__restr
     }
 }
 
+// ---- Pointer jumping of small trees by one block, in place in shared memory:
+// all steps in one launch (15 of them, some 2.5 us each, were most of the
+// orientation of a few thousand vertices; a step here is 0.5 us).  A step's new
+// values wait in registers for the barrier; PJ_PER elements a thread.
+constexpr int PJ_THREADS = 1024, PJ_PER = 16;
+constexpr int PJ_MAX = PJ_THREADS * PJ_PER;
+
+// list ranking (k_wyllie's steps and k_check_ranked), M <= PJ_MAX
+__global__ void __launch_bounds__(PJ_THREADS, 1) k_rank_small(const int32_t *__restrict__ succ, int32_t *__restrict__ rnk,
+                                                              int M, int steps, uint32_t *st) {
+    extern __shared__ int32_t pj[];
+    int32_t *ps = pj, *pr = pj + M;
+    const int tid = threadIdx.x;
+    for (int i = tid; i < M; i += PJ_THREADS) {
+        ps[i] = succ[i];
+        pr[i] = 1;
+    }
+    __syncthreads();
+    for (int it = 0; it < steps; ++it) {
+        int32_t s[PJ_PER], r[PJ_PER];
+#pragma unroll
+        for (int k = 0; k < PJ_PER; ++k) {
+            const int i = tid + k * PJ_THREADS;
+            s[k] = -1;
+            if (i < M) {
+                const int32_t q = ps[i];
+                r[k] = pr[i];
+                if (q >= 0) {
+                    r[k] += pr[q];
+                    s[k] = ps[q];
+                }
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < PJ_PER; ++k) {
+            const int i = tid + k * PJ_THREADS;
+            if (i < M) {
+                ps[i] = s[k];
+                pr[i] = r[k];
+            }
+        }
+        __syncthreads();
+    }
+    for (int i = tid; i < M; i += PJ_THREADS) {
+        rnk[i] = pr[i];
+        if (ps[i] != -1 || pr[i] < 1 || pr[i] > M) flag_status(st, DEV_BAD_TREE);
+    }
+}
+
+// depth and preorder (k_jump_acc's steps), n <= PJ_MAX
+__global__ void __launch_bounds__(PJ_THREADS, 1) k_jump_small(const int32_t *__restrict__ anc, int32_t *dep, int32_t *pre,
+                                                              int n, int steps) {
+    extern __shared__ int32_t pj[];
+    int32_t *pa = pj, *pd = pj + n, *pp = pj + 2 * n;
+    const int tid = threadIdx.x;
+    for (int i = tid; i < n; i += PJ_THREADS) {
+        pa[i] = anc[i];
+        pd[i] = dep[i];
+        pp[i] = pre[i];
+    }
+    __syncthreads();
+    for (int it = 0; it < steps; ++it) {
+        int32_t a[PJ_PER], x[PJ_PER], y[PJ_PER];
+        int left = 0;
+#pragma unroll
+        for (int k = 0; k < PJ_PER; ++k) {
+            const int i = tid + k * PJ_THREADS;
+            a[k] = -1;
+            x[k] = y[k] = 0;
+            if (i < n) {
+                const int32_t q = pa[i];
+                if (q >= 0) {
+                    x[k] = pd[q];
+                    y[k] = pp[q];
+                    a[k] = pa[q];
+                    left |= a[k] >= 0;
+                }
+            }
+        }
+        left = __syncthreads_or(left);
+#pragma unroll
+        for (int k = 0; k < PJ_PER; ++k) {
+            const int i = tid + k * PJ_THREADS;
+            if (i < n) {
+                pa[i] = a[k];
+                pd[i] += x[k];
+                pp[i] += y[k];
+            }
+        }
+        __syncthreads();
+        if (!left) break;                                // every pointer has passed the root
+    }
+    for (int i = tid; i < n; i += PJ_THREADS) {
+        dep[i] = pd[i];
+        pre[i] = pp[i];
+    }
+}
+
+// the ends of the pointer chains (k_head_jump's steps), n <= PJ_MAX
+__global__ void __launch_bounds__(PJ_THREADS, 1) k_head_small(int32_t *head, int n, int steps) {
+    extern __shared__ int32_t pj[];
+    const int tid = threadIdx.x;
+    for (int i = tid; i < n; i += PJ_THREADS) pj[i] = head[i];
+    __syncthreads();
+    for (int it = 0; it < steps; ++it) {
+        int32_t h[PJ_PER];
+        int moved = 0;
+#pragma unroll
+        for (int k = 0; k < PJ_PER; ++k) {
+            const int i = tid + k * PJ_THREADS;
+            if (i < n) {
+                const int32_t q = pj[i];
+                h[k] = pj[q];
+                moved |= h[k] != q;
+            }
+        }
+        moved = __syncthreads_or(moved);
+        if (!moved) break;
+#pragma unroll
+        for (int k = 0; k < PJ_PER; ++k) {
+            const int i = tid + k * PJ_THREADS;
+            if (i < n) pj[i] = h[k];
+        }
+        __syncthreads();
+    }
+    for (int i = tid; i < n; i += PJ_THREADS) head[i] = pj[i];
+}
+
+static cudaError_t pj_attr() {
+    static bool done = false;
+    if (done) return cudaSuccess;
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(k_rank_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * PJ_MAX))) return e;
+    if ((e = cudaFuncSetAttribute(k_jump_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 12 * PJ_MAX))) return e;
+    if ((e = cudaFuncSetAttribute(k_head_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * PJ_MAX))) return e;
+    done = true;
+    return cudaSuccess;
+}
+
 __global__ void k_check_ranked(const int32_t *__restrict__ succ, const int32_t *__restrict__ rnk,
                                int64_t M, uint32_t *st) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -972,12 +1112,12 @@ __global__ void __launch_bounds__(1024) k_cand_select(SearchState *S, uint32_t *
 // ---- Trees of at most SM_MAX_N vertices: one block per threshold evaluates
 // Algorithm 1 on the whole tree out of shared memory, level by level from the
 // deepest, in BFS order (a vertex's children are then contiguous).  A level
-// costs a barrier and a few shared-memory round trips (about 0.3 us) where a
+// costs a barrier and a few shared-memory round trips where a
 // step of the walks through global memory costs 2.5 us: 4,898 points (depth
 // 116) 0.28 ms a pass -> 0.04.  The block that finishes last updates the
 // search and picks the next thresholds, so a pass is one launch.  States go
 // out by [threshold][BFS position].
-constexpr int SM_THREADS = 512;
+constexpr int SM_THREADS = 512, SM_AHEAD = 4, SM_LEVELS = 1024;
 constexpr int SM_MAX_N = 12288;       // 17 bytes a vertex: 204 KB of shared memory
 constexpr int SM_MIN_SMEM = 2 * CAND_BUCKETS * (int)sizeof(uint32_t);
 inline int sm_smem(int64_t n) { return (int)(n * 17 > SM_MIN_SMEM ? n * 17 : SM_MIN_SMEM); }
@@ -1009,7 +1149,7 @@ __global__ void k_small_setup(SmallTree A, const int32_t *__restrict__ ch_off, c
     if (q == 0 || depth[A.order[q - 1]] != depth[v]) A.lstart[depth[v]] = q;
 }
 
-__global__ void __launch_bounds__(SM_THREADS) k_dp_small(SmallTree A, SearchState *S, int32_t k, int last, int final_pass,
+__global__ void __launch_bounds__(SM_THREADS, 1) k_dp_small(SmallTree A, SearchState *S, int32_t k, int last, int final_pass,
                                                          uint32_t *st) {
     if (!final_pass && S->done) return;
     if (final_pass && (S->final_lane >= 0 || blockIdx.x != 0)) return;      // (k_final_from_lane serves)
@@ -1018,6 +1158,7 @@ __global__ void __launch_bounds__(SM_THREADS) k_dp_small(SmallTree A, SearchStat
     double *W = reinterpret_cast<double *>(sm_raw), *P = W + n;
     uint8_t *Dc = reinterpret_cast<uint8_t *>(P + n);
     __shared__ int scuts, slast;
+    __shared__ int32_t slev[SM_LEVELS];                  // first position of the upper levels
     if (tid == 0) scuts = 0;
     const double N = final_pass ? S->beta : S->thr[t];
     uint8_t *gd = A.dec + (size_t)t * n;
@@ -1053,22 +1194,32 @@ __global__ void __launch_bounds__(SM_THREADS) k_dp_small(SmallTree A, SearchStat
         gw[q] = w;
         gp[q] = pv;
     };
-    // the next level's first vertices are on their way while a level is decided
-    int l = S->max_depth;
-    int s0 = A.lstart[l], e0 = n, s1 = l > 0 ? A.lstart[l - 1] : 0;
-    Vtx cur{}, nxt{};
-    if (s0 + tid < e0) cur = load(s0 + tid);
+    // A level is a few shared-memory round trips, its vertices' data an L2 one:
+    // the first vertices of the next SM_AHEAD levels are always on their way
+    // (one level ahead: 1.1 us a level at 4,898 points)
+    const int Lm = S->max_depth;
+    for (int l = tid; l < SM_LEVELS && l <= Lm; l += SM_THREADS) slev[l] = A.lstart[l];
     __syncthreads();
-    for (; l >= 0; --l) {
-        const int s2 = l > 1 ? A.lstart[l - 2] : 0;
-        if (l > 0 && s1 + tid < s0) nxt = load(s1 + tid);
-        if (s0 + tid < e0) decide(s0 + tid, cur);
-        for (int q = s0 + tid + SM_THREADS; q < e0; q += SM_THREADS) decide(q, load(q));
-        __syncthreads();
-        cur = nxt;
-        e0 = s0;
-        s0 = s1;
-        s1 = s2;
+    auto first = [&](int l) { return l > Lm ? n : (l < SM_LEVELS ? slev[l] : A.lstart[l]); };
+    Vtx buf[SM_AHEAD];
+    auto fetch = [&](int l, Vtx &x) {
+        if (l < 0) return;
+        const int q = first(l) + tid;
+        if (q < first(l + 1)) x = load(q);
+    };
+#pragma unroll
+    for (int u = 0; u < SM_AHEAD; ++u) fetch(Lm - u, buf[u]);
+    for (int l0 = Lm; l0 >= 0; l0 -= SM_AHEAD) {
+#pragma unroll
+        for (int u = 0; u < SM_AHEAD; ++u) {
+            const int l = l0 - u;
+            if (l < 0) break;
+            const int s0 = first(l), e0 = first(l + 1);
+            if (s0 + tid < e0) decide(s0 + tid, buf[u]);
+            for (int q = s0 + tid + SM_THREADS; q < e0; q += SM_THREADS) decide(q, load(q));
+            fetch(l - SM_AHEAD, buf[u]);
+            __syncthreads();
+        }
     }
     for (int o = 16; o > 0; o >>= 1) cuts += __shfl_xor_sync(0xffffffffu, cuts, o);
     if ((tid & 31) == 0 && cuts) atomicAdd(&scuts, cuts);
@@ -1105,19 +1256,38 @@ __global__ void __launch_bounds__(SM_THREADS) k_dp_small(SmallTree A, SearchStat
     if (!sact) return;
     const unsigned long long lo = slo, hi = shi;
     const double inv_w = (double)CAND_BUCKETS / (double)(hi - lo);
-    auto add = [&](double c) {
-        const unsigned long long b = dbits(c);
-        if (!(c > 0.0) || b <= lo || b >= hi) return;
+    // FP64 quotients of all vertices on one SM are some 50 us at 4,898 points,
+    // so FP32 ones sort out first what lies outside the bracket, and while
+    // that is wide (the counts only place thresholds then) they also pick the
+    // bucket.  FP32's error: two conversions and a quotient of 2 units.
+    const float lof = (float)bitsd(lo), hif = (float)bitsd(hi), slack = 1e-6f;
+    const bool wide = bitsd(hi) > bitsd(lo) * 1.01;
+    auto tame = [](float x) { return x > 1e-18f && x < 1e18f; };
+    auto add = [&](double num, double w) {
+        if (!(num > 0.0)) return;
+        const float nf = (float)num, wf = (float)w;
+        unsigned long long b = 0ull;
+        bool have = false;
+        if (tame(nf) && tame(wf) && tame(lof) && tame(hif)) {
+            const float qf = nf / wf;
+            if (qf < lof * (1.0f - slack) || qf > hif * (1.0f + slack)) return;
+            have = wide && qf > lof * (1.0f + slack) && qf < hif * (1.0f - slack);
+            if (have) b = dbits((double)qf);
+        }
+        if (!have) {
+            b = dbits(__ddiv_rn(num, w));
+            if (b <= lo || b >= hi) return;
+        }
         atomicAdd(hist + cand_bucket(b, lo, inv_w), 1u);
         const unsigned q = atomicAdd(&snc, 1u);
-        if (q < (unsigned)CAND_EXACT) scand[q] = b;
+        if (q < (unsigned)CAND_EXACT) scand[q] = have ? dbits(__ddiv_rn(num, w)) : b;
     };
     const double *lw = A.wh + (size_t)sL * n, *lp = A.ph + (size_t)sL * n;
     for (int q = tid; q < n; q += SM_THREADS) {
         const double w = ld_cg_f64(lw + q), pv = ld_cg_f64(lp + q);
         const double fe = q > 0 ? A.phi[q] : 0.0;
-        add(__ddiv_rn(__dadd_rn(fe, pv), w));
-        if (q > 0) add(__ddiv_rn(__dsub_rn(pv, fe), w));
+        add(__dadd_rn(fe, pv), w);
+        if (q > 0) add(__dsub_rn(pv, fe), w);
     }
     __syncthreads();
     cand_select_block<SM_THREADS>(S, hist, pre, snc, scand);
@@ -1425,6 +1595,9 @@ cudaError_t orient_tree(TreeScratch &S, const int32_t *eu, const int32_t *ev, in
     const int L = log2_ceil(M) + 1;
     // the ranks end in rnk after an even number of Wyllie steps, else rnk2
     int32_t *ra = (L % 2 == 0) ? S.rnk : S.rnk2;
+    const bool rank_small = M <= PJ_MAX;
+    if (rank_small) ra = S.rnk;
+    if ((e = pj_attr())) return e;
     if (part != 2) {
         k_dir_keys<<<blocks_for(m), TPB, 0, ISO_S(s)>>>(eu, ev, m, n, T.adj_key, S.vals, S.status);
         if ((e = sort_pairs_u64(T.adj_key, S.vals, S.kbuf, S.vbuf, M, s))) return e;
@@ -1433,14 +1606,18 @@ cudaError_t orient_tree(TreeScratch &S, const int32_t *eu, const int32_t *ev, in
         k_check_adj<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(T.adj_off, n, S.status);
         k_rev_succ<<<blocks_for(M), TPB, 0, ISO_S(s)>>>(T.adj_key, T.adj_off, M, n, S.rev, S.succ, S.status);
         k_break_tour<<<1, 1, 0, ISO_S(s)>>>(T.adj_off, S.rev, S.succ, root, M, S.status);
-        k_fill_i32<<<blocks_for(M), TPB, 0, ISO_S(s)>>>(S.rnk, M, 1);
-        int32_t *sa = S.succ, *sb = S.succ2, *rk = S.rnk, *rb = S.rnk2;
-        for (int it = 0; it < L; ++it) {
-            k_wyllie<<<blocks_for(M), TPB, 0, ISO_S(s)>>>(sa, rk, sb, rb, M);
-            int32_t *t = sa; sa = sb; sb = t;
-            t = rk; rk = rb; rb = t;
+        if (rank_small) {
+            k_rank_small<<<1, PJ_THREADS, (size_t)M * 8, ISO_S(s)>>>(S.succ, S.rnk, (int)M, L, S.status);
+        } else {
+            k_fill_i32<<<blocks_for(M), TPB, 0, ISO_S(s)>>>(S.rnk, M, 1);
+            int32_t *sa = S.succ, *sb = S.succ2, *rk = S.rnk, *rb = S.rnk2;
+            for (int it = 0; it < L; ++it) {
+                k_wyllie<<<blocks_for(M), TPB, 0, ISO_S(s)>>>(sa, rk, sb, rb, M);
+                int32_t *t = sa; sa = sb; sb = t;
+                t = rk; rk = rb; rb = t;
+            }
+            k_check_ranked<<<blocks_for(M), TPB, 0, ISO_S(s)>>>(sa, rk, M, S.status);
         }
-        k_check_ranked<<<blocks_for(M), TPB, 0, ISO_S(s)>>>(sa, rk, M, S.status);
         if (part == 1) return cudaGetLastError();
         uint32_t hst = 0;
         if ((e = cudaMemcpyAsync(&hst, S.status, sizeof(uint32_t), cudaMemcpyDeviceToHost, s))) return e;
@@ -1459,16 +1636,21 @@ cudaError_t orient_tree(TreeScratch &S, const int32_t *eu, const int32_t *ev, in
     k_child_sizes<<<blocks_for(m), TPB, 0, ISO_S(s)>>>(T.ch_list, S.size, m, S.ssz);
     if ((e = exclusive_scan_i64(S.ssz, S.sx, m, S.tmp64, s))) return e;
     k_pre_init<<<blocks_for(m), TPB, 0, ISO_S(s)>>>(T.parent, T.ch_off, T.ch_list, S.sx, m, root, S.anc, T.depth, S.pre);
-    int32_t *aa = S.anc, *ab = S.anc2, *da = T.depth, *db = S.dep2, *pa = S.pre, *pb = S.pre2;
     const int Ln = log2_ceil(n) + 1;
-    for (int it = 0; it < Ln; ++it) {
-        k_jump_acc<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(aa, da, pa, ab, db, pb, n);
-        int32_t *t = aa; aa = ab; ab = t;
-        t = da; da = db; db = t;
-        t = pa; pa = pb; pb = t;
-    }
-    if (da != T.depth) {
-        if ((e = cudaMemcpyAsync(T.depth, da, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s))) return e;
+    int32_t *pa = S.pre;
+    if (n <= PJ_MAX) {
+        k_jump_small<<<1, PJ_THREADS, (size_t)n * 12, ISO_S(s)>>>(S.anc, T.depth, S.pre, (int)n, Ln);
+    } else {
+        int32_t *aa = S.anc, *ab = S.anc2, *da = T.depth, *db = S.dep2, *pb = S.pre2;
+        for (int it = 0; it < Ln; ++it) {
+            k_jump_acc<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(aa, da, pa, ab, db, pb, n);
+            int32_t *t = aa; aa = ab; ab = t;
+            t = da; da = db; db = t;
+            t = pa; pa = pb; pb = t;
+        }
+        if (da != T.depth) {
+            if ((e = cudaMemcpyAsync(T.depth, da, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s))) return e;
+        }
     }
     T.pre = pa;
     k_bfs_keys<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(T.depth, pa, n, S.bkeys, S.ib);
@@ -1582,9 +1764,14 @@ cudaError_t tree_search_and_label(TreeScratch &S, const double *phi_par, const d
     k_head_init<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, slot, sv, T.parent, n, S.head);
     int32_t *ha = S.head, *hb = S.head2;
     const int Ln = log2_ceil(n) + 1;
-    for (int it = 0; it < Ln; ++it) {
-        k_head_jump<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(ha, hb, n);
-        int32_t *t = ha; ha = hb; hb = t;
+    if (n <= PJ_MAX) {
+        if ((e = pj_attr())) return e;
+        k_head_small<<<1, PJ_THREADS, (size_t)n * 4, ISO_S(s)>>>(S.head, (int)n, Ln);
+    } else {
+        for (int it = 0; it < Ln; ++it) {
+            k_head_jump<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(ha, hb, n);
+            int32_t *t = ha; ha = hb; hb = t;
+        }
     }
     k_cut_flags<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, slot, sv, T.bfs_pos, n, S.cflag);
     if ((e = exclusive_scan_i32(S.cflag, S.cidx, n, S.tmp32, s))) return e;
@@ -1634,9 +1821,14 @@ cudaError_t tree_search_and_label_sets(TreeScratch &S, int32_t nsets, const int6
     k_head_init<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, nullptr, DP_LANES, T.parent, n, S.head);
     int32_t *ha = S.head, *hb = S.head2;
     const int Ln = log2_ceil(n) + 1;
-    for (int it = 0; it < Ln; ++it) {
-        k_head_jump<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(ha, hb, n);
-        int32_t *t = ha; ha = hb; hb = t;
+    if (n <= PJ_MAX) {
+        if ((e = pj_attr())) return e;
+        k_head_small<<<1, PJ_THREADS, (size_t)n * 4, ISO_S(s)>>>(S.head, (int)n, Ln);
+    } else {
+        for (int it = 0; it < Ln; ++it) {
+            k_head_jump<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(ha, hb, n);
+            int32_t *t = ha; ha = hb; hb = t;
+        }
     }
     k_cut_flags<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(S.dec, nullptr, DP_LANES, T.bfs_pos, n, S.cflag);
     if ((e = exclusive_scan_i32(S.cflag, S.cidx, n, S.tmp32, s))) return e;
