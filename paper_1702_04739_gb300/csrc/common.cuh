@@ -1,6 +1,7 @@
 // common.cuh -- shared internals of the isoclust CUDA library (sm_103a).
 #pragma once
 
+#include <atomic>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stddef.h>
@@ -87,6 +88,19 @@ struct Arena {
         return reinterpret_cast<T *>(base + a);
     }
 };
+
+// Whether this is the first time for the caller's flags on the current device
+// (function attributes are per device; setting one twice does no harm).
+inline bool first_on_device(std::atomic<unsigned long long> &seen) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return true;
+    const unsigned long long bit = 1ull << (dev & 63);
+    return !(seen.load(std::memory_order_acquire) & bit);
+}
+inline void done_on_device(std::atomic<unsigned long long> &seen) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) seen.fetch_or(1ull << (dev & 63), std::memory_order_release);
+}
 
 // Per-device cached scratch (grow-only).  Returns nullptr on failure.
 void *scratch_acquire(size_t bytes, cudaStream_t stream, isoclust_status *st);

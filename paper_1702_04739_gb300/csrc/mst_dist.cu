@@ -108,26 +108,19 @@ __global__ void __launch_bounds__(256) k_dist_tiles(const P *__restrict__ X, int
     }
 }
 
-// One row per block.  DK_INLINE (short rows): a thread keys its own columns, the
-// block's best goes to rowd2 / rowj and to its component's minimum.  DK_SPARSE:
-// the same from the rows' non-zeros (a dimension that neither row holds adds
-// nothing to the key); the distances come from a Gram, within err (|x_i|^2 +
-// |x_j|^2) of the true ones.  DK_LIST: the columns go to surv for the FP64 keys
-// of long rows, more than SURV of them (exact ties) to the rescan.
-// A thread whose own columns hold none within the margin does not look again:
-// of long rows (512 threads) the second look reads a tenth of the matrix.
-constexpr int DSC_SURV = 8;
-enum : int { DK_INLINE = 0, DK_LIST = 1, DK_SPARSE = 2 };
-template <class P, int KIND, int DSC_THREADS>
+// One row per block.  INLINE (short rows): a thread keys its own columns, the
+// block's best goes to rowd2 / rowj and to its component's minimum.  Else the
+// columns go to surv for the FP64 keys of long rows, more than SURV of them
+// (exact ties) to the rescan.
+constexpr int DSC_THREADS = 128, DSC_SURV = 8;
+template <class P, bool INLINE>
 __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__ X, int64_t n, int32_t d,
                                                            const float *__restrict__ D, int64_t ld, float mul, float add,
                                                            const int32_t *__restrict__ comp, double *__restrict__ rowd2,
                                                            int32_t *__restrict__ rowj, unsigned long long *__restrict__ cd2,
                                                            int32_t *__restrict__ nsurv, int32_t *__restrict__ surv,
-                                                           int32_t *__restrict__ ovf, int32_t *counters,
-                                                           const SparseRows R, float err) {
+                                                           int32_t *__restrict__ ovf, int32_t *counters) {
     if (!dist_active(counters)) return;
-    constexpr bool INLINE = KIND != DK_LIST;
     __shared__ float smin[DSC_THREADS / 32];
     __shared__ double sb[DSC_THREADS / 32];
     __shared__ int32_t sj[DSC_THREADS / 32];
@@ -136,27 +129,19 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
     const int64_t i = blockIdx.x;
     const int32_t ci = comp[i];
     const float *row = D + i * ld;
-    // the largest and the smallest distance that an entry stands for
-    const float ni = KIND == DK_SPARSE ? R.norm[i].x : 0.0f;
-    auto wide = [&](int64_t j) { return __fmul_ru(err, __fadd_ru(ni, R.norm[j].x)); };
-    auto up = [&](float v, int64_t j) { return KIND == DK_SPARSE ? __fadd_ru(v, wide(j)) : v; };
-    auto down = [&](float v, int64_t j) { return KIND == DK_SPARSE ? __fsub_rd(v, wide(j)) : v; };
     const int64_t n4 = n & ~(int64_t)3;
     if (tid == 0) scnt = 0;
-    float m = INFINITY, low = INFINITY;
-    auto first = [&](float v, int64_t j) {
-        m = fminf(m, up(v, j));
-        low = fminf(low, down(v, j));
-    };
+    float m = INFINITY;
     for (int64_t j = 4 * tid; j < n4; j += 4 * DSC_THREADS) {
         const float4 v = *reinterpret_cast<const float4 *>(row + j);
         const int4 c = *reinterpret_cast<const int4 *>(comp + j);
-        if (c.x != ci) first(v.x, j);
-        if (c.y != ci) first(v.y, j + 1);
-        if (c.z != ci) first(v.z, j + 2);
-        if (c.w != ci) first(v.w, j + 3);
+        if (c.x != ci) m = fminf(m, v.x);
+        if (c.y != ci) m = fminf(m, v.y);
+        if (c.z != ci) m = fminf(m, v.z);
+        if (c.w != ci) m = fminf(m, v.w);
     }
-    if (n4 + tid < n && comp[n4 + tid] != ci) first(row[n4 + tid], n4 + tid);
+    if (n4 + tid < n && comp[n4 + tid] != ci) m = fminf(m, row[n4 + tid]);
+    const float low = m;                   // (a thread whose own columns hold none does not look again)
     for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) smin[wp] = m;
     __syncthreads();
@@ -168,21 +153,9 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
     auto see = [&](int64_t j) {
         if constexpr (INLINE) {
             double e = 0.0;
-            if constexpr (KIND == DK_SPARSE) {
-                int32_t a = R.rowptr[i], b = R.rowptr[j];
-                const int32_t a1 = R.rowptr[i + 1], b1 = R.rowptr[j + 1];
-                while (a < a1 || b < b1) {
-                    const int32_t ta = a < a1 ? R.rcol[a] : INT32_MAX, tb = b < b1 ? R.rcol[b] : INT32_MAX;
-                    double df = 0.0;
-                    if (ta <= tb) df = (double)R.rval[a++];
-                    if (tb <= ta) df = __dsub_rn(df, (double)R.rval[b++]);
-                    e = __dadd_rn(e, __dmul_rn(df, df));
-                }
-            } else {
-                for (int t = 0; t < d; ++t) {
-                    const double df = __dsub_rn((double)X[i * d + t], (double)X[j * d + t]);
-                    e = __dadd_rn(e, __dmul_rn(df, df));
-                }
+            for (int t = 0; t < d; ++t) {
+                const double df = __dsub_rn((double)X[i * d + t], (double)X[j * d + t]);
+                e = __dadd_rn(e, __dmul_rn(df, df));
             }
             if (bestj < 0 || key_less(e, (int32_t)i, (int32_t)j, best, (int32_t)i, bestj)) {
                 best = e;
@@ -196,14 +169,14 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
     if (low <= thr)
         for (int64_t j = 4 * tid; j < n4; j += 4 * DSC_THREADS) {
             const float4 v = *reinterpret_cast<const float4 *>(row + j);
-            if (KIND != DK_SPARSE && fminf(fminf(v.x, v.y), fminf(v.z, v.w)) > thr) continue;
+            if (fminf(fminf(v.x, v.y), fminf(v.z, v.w)) > thr) continue;
             const int4 c = *reinterpret_cast<const int4 *>(comp + j);
-            if (c.x != ci && down(v.x, j) <= thr) see(j);
-            if (c.y != ci && down(v.y, j + 1) <= thr) see(j + 1);
-            if (c.z != ci && down(v.z, j + 2) <= thr) see(j + 2);
-            if (c.w != ci && down(v.w, j + 3) <= thr) see(j + 3);
+            if (c.x != ci && v.x <= thr) see(j);
+            if (c.y != ci && v.y <= thr) see(j + 1);
+            if (c.z != ci && v.z <= thr) see(j + 2);
+            if (c.w != ci && v.w <= thr) see(j + 3);
         }
-    if (n4 + tid < n && comp[n4 + tid] != ci && down(row[n4 + tid], n4 + tid) <= thr) see(n4 + tid);
+    if (n4 + tid < n && comp[n4 + tid] != ci && row[n4 + tid] <= thr) see(n4 + tid);
     if constexpr (INLINE) {
         auto take = [&](double e, int32_t j) {
             if (j >= 0 && (bestj < 0 || key_less(e, (int32_t)i, j, best, (int32_t)i, bestj))) {
@@ -237,6 +210,185 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
                 rowj[i] = -2;
             }
         }
+    }
+}
+
+// The scan for rows as lists: the distances come from a Gram, within err (|x_i|^2
+// + |x_j|^2) of the true ones, so a column is a candidate when the smallest
+// distance its entry stands for is at most the smallest of the row's largest.
+// Keys from the lists (a dimension that neither row holds adds nothing to the
+// key), by a warp per candidate: the lanes find each entry's place in the two
+// lists' common order and leave its square there, one adds them up.  (One
+// thread walking the lists, in global or in shared memory: some 10 us of
+// latency a key, 6 ms a round at 50,000 x 4,096.)  Only a thread whose own
+// columns hold two candidates or more looks at them again.
+constexpr int SC_THREADS = 512, SC_CAND = 128, SC_LIST = 128;
+__global__ void __launch_bounds__(SC_THREADS) k_sparse_scan(const SparseRows R, int64_t n, const float *__restrict__ D,
+                                                            int64_t ld, float err, float add,
+                                                            const int32_t *__restrict__ comp, double *__restrict__ rowd2,
+                                                            int32_t *__restrict__ rowj,
+                                                            unsigned long long *__restrict__ cd2, const int32_t *counters) {
+    if (!dist_active(counters)) return;
+    constexpr int NW = SC_THREADS / 32;
+    __shared__ float smin[NW];
+    __shared__ double sb[NW];
+    __shared__ int32_t sj[NW], scand[SC_CAND];
+    __shared__ int scnt;
+    __shared__ int32_t ac[SC_LIST], bc[NW][SC_LIST];
+    __shared__ float av[SC_LIST], bv[NW][SC_LIST];
+    __shared__ double sq[NW][2 * SC_LIST];
+    const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+    const int64_t i = blockIdx.x;
+    const int32_t ci = comp[i];
+    const float *row = D + i * ld;
+    const float ni = R.norm1[i];
+    const int32_t a0 = R.rowptr[i], alen = R.rowptr[i + 1] - a0;
+    for (int e = tid; e < alen && e < SC_LIST; e += SC_THREADS) {
+        ac[e] = R.rcol[a0 + e];
+        av[e] = R.rval[a0 + e];
+    }
+    if (tid == 0) scnt = 0;
+    const int64_t n4 = n & ~(int64_t)3;
+    auto wide = [&](float nj) { return __fmul_ru(err, __fadd_ru(ni, nj)); };
+    // the thread's two smallest, and the column of the smaller
+    float m = INFINITY, low = INFINITY, low2 = INFINITY;
+    int32_t lowj = -1;
+    auto first = [&](float v, float nj, int64_t j) {
+        const float w = wide(nj), l = __fsub_rd(v, w);
+        m = fminf(m, __fadd_ru(v, w));
+        low2 = fminf(low2, fmaxf(low, l));
+        if (l < low) {
+            low = l;
+            lowj = (int32_t)j;
+        }
+    };
+#pragma unroll 4
+    for (int64_t j = 4 * tid; j < n4; j += 4 * SC_THREADS) {
+        const float4 v = *reinterpret_cast<const float4 *>(row + j);
+        const int4 c = *reinterpret_cast<const int4 *>(comp + j);
+        const float4 q = *reinterpret_cast<const float4 *>(R.norm1 + j);
+        if (c.x != ci) first(v.x, q.x, j);
+        if (c.y != ci) first(v.y, q.y, j + 1);
+        if (c.z != ci) first(v.z, q.z, j + 2);
+        if (c.w != ci) first(v.w, q.w, j + 3);
+    }
+    if (n4 + tid < n && comp[n4 + tid] != ci) first(row[n4 + tid], R.norm1[n4 + tid], n4 + tid);
+    for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) smin[wp] = m;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NW; ++q) m = fminf(m, smin[q]);
+    const float thr = __fadd_ru(m, add);
+    double best = INFINITY;
+    int32_t bestj = -1;
+    auto take = [&](double e, int32_t j) {
+        if (j >= 0 && (bestj < 0 || key_less(e, (int32_t)i, j, best, (int32_t)i, bestj))) {
+            best = e;
+            bestj = j;
+        }
+    };
+    // the key along two lists, smallest dimension first
+    auto key = [&](const int32_t *xc, const float *xv, int xn, const int32_t *yc, const float *yv, int yn) {
+        double e = 0.0;
+        int a = 0, b = 0;
+        int32_t ta = xn > 0 ? xc[0] : INT32_MAX, tb = yn > 0 ? yc[0] : INT32_MAX;
+        while (a < xn || b < yn) {
+            double df = 0.0;
+            const bool ua = ta <= tb, ub = tb <= ta;
+            if (ua) {
+                df = (double)xv[a++];
+                ta = a < xn ? xc[a] : INT32_MAX;
+            }
+            if (ub) {
+                df = __dsub_rn(df, (double)yv[b++]);
+                tb = b < yn ? yc[b] : INT32_MAX;
+            }
+            e = __dadd_rn(e, __dmul_rn(df, df));
+        }
+        return e;
+    };
+    auto see = [&](int64_t j) {
+        const int q = atomicAdd(&scnt, 1);
+        if (q < SC_CAND) {
+            scand[q] = (int32_t)j;
+        } else {                                         // (many ties: by the thread itself)
+            const int32_t b0 = R.rowptr[j];
+            take(key(R.rcol + a0, R.rval + a0, alen, R.rcol + b0, R.rval + b0, R.rowptr[j + 1] - b0), (int32_t)j);
+        }
+    };
+    auto again = [&](float v, float nj, int32_t c, int64_t j) {
+        if (c != ci && __fsub_rd(v, wide(nj)) <= thr) see(j);
+    };
+    if (low <= thr && low2 > thr) {
+        see(lowj);
+    } else if (low <= thr) {
+        for (int64_t j = 4 * tid; j < n4; j += 4 * SC_THREADS) {
+            const float4 v = *reinterpret_cast<const float4 *>(row + j);
+            const int4 c = *reinterpret_cast<const int4 *>(comp + j);
+            const float4 q = *reinterpret_cast<const float4 *>(R.norm1 + j);
+            again(v.x, q.x, c.x, j);
+            again(v.y, q.y, c.y, j + 1);
+            again(v.z, q.z, c.z, j + 2);
+            again(v.w, q.w, c.w, j + 3);
+        }
+        if (n4 + tid < n) again(row[n4 + tid], R.norm1[n4 + tid], comp[n4 + tid], n4 + tid);
+    }
+    __syncthreads();
+    const int nc = scnt < SC_CAND ? scnt : SC_CAND;
+    for (int q = wp; q < nc; q += NW) {
+        const int32_t j = scand[q], b0 = R.rowptr[j], blen = R.rowptr[j + 1] - b0;
+        const bool fits = alen <= SC_LIST && blen <= SC_LIST;
+        __syncwarp();
+        if (fits)
+            for (int e = lane; e < blen; e += 32) {
+                bc[wp][e] = R.rcol[b0 + e];
+                bv[wp][e] = R.rval[b0 + e];
+            }
+        __syncwarp();
+        if (fits) {
+            // entries of a list below t (or up to it)
+            auto below = [](const int32_t *l, int n_, int32_t t) {
+                int lo = 0, hi = n_;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (l[mid] < t) lo = mid + 1; else hi = mid;
+                }
+                return lo;
+            };
+            for (int e = lane; e < alen; e += 32) {
+                const int p = below(bc[wp], blen, ac[e]);
+                const double df = p < blen && bc[wp][p] == ac[e] ? __dsub_rn((double)av[e], (double)bv[wp][p]) : (double)av[e];
+                sq[wp][e + p] = __dmul_rn(df, df);
+            }
+            for (int e = lane; e < blen; e += 32) {
+                const int p = below(ac, alen, bc[wp][e] + 1);       // a dimension of both: the other list's entry, then a zero
+                const bool both = p > 0 && ac[p - 1] == bc[wp][e];
+                const double df = (double)bv[wp][e];
+                sq[wp][e + p] = both ? 0.0 : __dmul_rn(df, df);
+            }
+            __syncwarp();
+            double e = 0.0;
+            for (int k = 0; k < alen + blen; ++k) e = __dadd_rn(e, sq[wp][k]);
+            if (lane == 0) take(e, j);
+        } else if (lane == 0) {
+            take(key(R.rcol + a0, R.rval + a0, alen, R.rcol + b0, R.rval + b0, blen), j);
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const double e = __shfl_xor_sync(0xffffffffu, best, o);
+        const int32_t j = __shfl_xor_sync(0xffffffffu, bestj, o);
+        take(e, j);
+    }
+    if (lane == 0) {
+        sb[wp] = best;
+        sj[wp] = bestj;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        for (int q = 1; q < NW; ++q) take(sb[q], sj[q]);
+        rowd2[i] = best;
+        rowj[i] = bestj;
+        if (bestj >= 0) atomicMin(cd2 + ci, dbits(best));
     }
 }
 
@@ -398,32 +550,31 @@ cudaError_t mst_build_dist(MstScratch &S, TcScratch &T, float *D, const void *X,
     // any column within m (1 + e) / (1 - e) + 2 add of the row's FP32 minimum
     // can hold the exact best (e: 10 % above the bound of the distances)
     const double u = 5.9604644775390625e-08, er = 1.1 * (double)(d + 3) * u;
-    const double mul = sp ? 1.0 : (1.0 + er) / (1.0 - er), add = (double)(d + 1) * 1.401298464324817e-45 * 4.0;
+    const double mul = (1.0 + er) / (1.0 - er), add = (double)(d + 1) * 1.401298464324817e-45 * 4.0;
     const float mul32 = (float)(mul * (1.0 + 1e-6)), add32 = (float)(2.01 * add) + 1.401298464324817e-45f;
     // A Gram's distance: the products' sums (a rounding per entry of the shorter
     // row, 2^-24 of |x_i| |x_j| <= (|x_i|^2 + |x_j|^2) / 2 each, twice), the norms
     // and the two last operations: within (longest + 5) 2^-24 (|x_i|^2 + |x_j|^2)
     const float err = sp ? (float)(1.1 * (double)(longest + 6) * u) : 0.0f;
-    const SparseRows none, &R0 = sp ? *sp : none;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if ((e = cudaStreamIsCapturing(s, &cs))) return e;
     const bool ask = cs == cudaStreamCaptureStatusNone;
     int R = 1;                                         // components at least halve per round
     while ((int64_t(1) << (R - 1)) < n) ++R;
     for (int r = 0; r < R; ++r) {
-#define ISO_SCAN(PT, KIND, NT)                                                                                            \
-    k_dist_scan<PT, KIND, NT><<<(unsigned)n, NT, 0, ISO_S(s)>>>((const PT *)X, n, d, D, ld, mul32, add32, S.comp,   \
+#define ISO_SCAN(PT, INL)                                                                                              \
+    k_dist_scan<PT, INL><<<(unsigned)n, DSC_THREADS, 0, ISO_S(s)>>>((const PT *)X, n, d, D, ld, mul32, add32, S.comp,   \
                                                                     S.rowd2, S.rowj, S.cd2, T.nsurv, T.surv,           \
-                                                                    S.ovf_rows, S.counters, R0, err)
+                                                                    S.ovf_rows, S.counters)
         if (sp) {
-            if (n > MST_DIST_MAX_N) ISO_SCAN(float, DK_SPARSE, 512);
-            else ISO_SCAN(float, DK_SPARSE, 128);
+            k_sparse_scan<<<(unsigned)n, SC_THREADS, 0, ISO_S(s)>>>(*sp, n, D, ld, err, add32, S.comp, S.rowd2, S.rowj, S.cd2,
+                                                                   S.counters);
         } else if (f64) {
-            ISO_SCAN(double, DK_INLINE, 128);
+            ISO_SCAN(double, true);
         } else if (inl) {
-            ISO_SCAN(float, DK_INLINE, 128);
+            ISO_SCAN(float, true);
         } else {
-            ISO_SCAN(float, DK_LIST, 128);
+            ISO_SCAN(float, false);
             if ((e = tc_key_rows(T, S, (const float *)X, n, d, mul, add, s))) return e;
             if ((e = mst_component_minima(S, n, s))) return e;
         }

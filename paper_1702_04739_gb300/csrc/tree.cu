@@ -322,13 +322,13 @@ __global__ void __launch_bounds__(PJ_THREADS, 1) k_head_small(int32_t *head, int
 }
 
 static cudaError_t pj_attr() {
-    static bool done = false;
-    if (done) return cudaSuccess;
+    static std::atomic<unsigned long long> seen{0};
+    if (!first_on_device(seen)) return cudaSuccess;
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(k_rank_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * PJ_MAX))) return e;
     if ((e = cudaFuncSetAttribute(k_jump_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 12 * PJ_MAX))) return e;
     if ((e = cudaFuncSetAttribute(k_head_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * PJ_MAX))) return e;
-    done = true;
+    done_on_device(seen);
     return cudaSuccess;
 }
 
@@ -1715,11 +1715,11 @@ cudaError_t tree_search_and_label(TreeScratch &S, const double *phi_par, const d
         A.ph = S.ph;
         A.rat = S.rat;
         const int smem = sm_smem(n);
-        static bool attr = false;
-        if (!attr) {
+        static std::atomic<unsigned long long> seen{0};
+        if (first_on_device(seen)) {
             if ((e = cudaFuncSetAttribute(k_dp_small, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_smem(SM_MAX_N))))
                 return e;
-            attr = true;
+            done_on_device(seen);
         }
         k_small_setup<<<blocks_for(n), TPB, 0, ISO_S(s)>>>(A, T.ch_off, T.ch_list, T.bfs_pos, T.depth, phi_par, omega, p);
         for (int pass = 0; pass < DP_TREE_PASSES; ++pass) {
