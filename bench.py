@@ -254,14 +254,17 @@ def omega_fused_roofline(prof, peaks, src, alu_peak, sms, kernel_ms, items, d, a
     blocks, direct = prof[-1]["omega_gram_blocks"], prof[-1].get("omega_gram_direct_pairs", 0)
     seconds = kernel_ms / 1000.0
     bf16 = peaks.get("bf16_tflops", 1900.0)
-    tc = blocks * 34 * 2.0 * 128 * 64 * (-(-d // 16) * 16) / seconds / 1e12
+    # rows with few non-zeros (long rows whose tree took no tensor-core sweep): the Gram from their lists, no MMAs
+    lists = d >= 512 and not prof[-1].get("mst_tiles_full", 1)
+    tc = 0.0 if lists else blocks * 34 * 2.0 * 128 * 64 * (-(-d // 16) * 16) / seconds / 1e12
     alu = (items * 4096.0 * 147.0 + direct * (18.75 * d + 95.0)) / seconds / 1e12
     alg = alg_flop / seconds / 1e12
     tensor = {"bound": "tensor", "achieved": tc, "peak": bf16, "frac": tc / bf16, "blocks": blocks}
     vector = {"bound": "alu", "achieved": alu, "peak": alu_peak, "frac": alu / alu_peak, "direct_pairs": direct,
               "direct_share": direct / max(1.0, items * 4096.0)}
     top, other = (tensor, vector) if tc / bf16 > alu / alu_peak else (vector, tensor)
-    return dict(top, unit="TFLOP/s", kernel="k_omega_tc (omega, Gram on tcgen05 and double-word FP32 terms)",
+    return dict(top, unit="TFLOP/s", kernel=f"k_omega_tc (omega, Gram {'from the rows lists' if lists else 'on tcgen05'} and double-word FP32 "
+                             "terms)",
                 kernel_ms=kernel_ms, traffic=None, other_unit=other,
                 note=f"FP32-pipe instructions of the algorithm as built (147 per pair of the {items} kept 64x64 tile "
                      f"pairs, 18.75 d + 95 per direct pair) over {sms} SMs x {FP32_LANES_PER_SM} lanes x max SM clock "
@@ -323,18 +326,20 @@ def omega_gram_roofline(prof, peaks, src, alu_peak, sms, sweep_ms, items, d, alg
     return out
 
 
-def mst_summary(prof, n_pairs_alg, pad_pairs_exe, d, sweep_variant):
+def mst_summary(prof, n_pairs_alg, pad_pairs_exe, d, sweep_variant, sets=False):
     """MST stage: the brute-force Boruvka Gram work (n(n-1)/2 pairs x 2d
     flop per round) and the tensor-core MMAs as issued (3 BF16 products over
     the 128 x 128 tile pairs actually swept: all of them per round without
-    pruning), both against the measured BF16 peak."""
+    pruning), both against the measured BF16 peak.  A tree on stored
+    distances (sweep_variant -1) issues no MMAs; independent sets sweep every
+    tile pair of every round."""
     peaks, src = _peaks()
     peak = peaks.get("bf16_tflops", 1900.0)
     mst_ms = statistics.mean(p["mst_ms"] for p in prof)
     rounds = prof[-1]["boruvka_rounds"]
     d_pad = -(-d // 64) * 64
-    swept, full = prof[-1].get("mst_tiles_swept", 0), prof[-1].get("mst_tiles_full", 0)
-    tile_pairs = swept if full else rounds * pad_pairs_exe / (128.0 * 128.0)
+    swept, full = (0, 0) if sets else (prof[-1].get("mst_tiles_swept", 0), prof[-1].get("mst_tiles_full", 0))
+    tile_pairs = swept if full else (0.0 if sweep_variant < 0 else rounds * pad_pairs_exe / (128.0 * 128.0))
     alg = rounds * n_pairs_alg * 2.0 * d / (mst_ms / 1000.0) / 1e12
     exe = 3 * 2.0 * tile_pairs * 128.0 * 128.0 * d_pad / (mst_ms / 1000.0) / 1e12
     return {"stage_ms": mst_ms, "rounds": rounds, "sweep_variant": sweep_variant,
@@ -455,7 +460,7 @@ def measure_batched(torch, dev, X, offs, ks, sigma, steps, warmup, pg=None, worl
     pairs = float((sizes * (sizes - 1) / 2).sum())
     out["roofline"] = omega_roofline(torch, dev, prof, pairs, d, BATCHED, sets=True)
     pad = -(-sizes // 128) * 128
-    out["mst"] = mst_summary(prof, pairs, float((pad ** 2).sum()), d, isoclust.last_sweep_variant())
+    out["mst"] = mst_summary(prof, pairs, float((pad ** 2).sum()), d, isoclust.last_sweep_variant(), sets=True)
     out["stages_ms"] = _stages(prof)
     detail = None
     if want_detail:
