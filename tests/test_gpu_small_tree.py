@@ -1,6 +1,7 @@
 """The search of a tree of up to 12,288 vertices (a block per threshold, the
 tree in shared memory) at the ends of its range and against the larger trees'
-passes: the oracle's i_k, labels and residual, with and without potentials."""
+passes, and the pointer jumping of up to 16,384 elements by one block: the
+oracle's i_k, labels and residual, with and without potentials."""
 import numpy as np
 import pytest
 
@@ -17,7 +18,7 @@ def iso():
     return isoclust
 
 
-@pytest.mark.parametrize("n", [2, 3, 511, 512, 513, 4898, 12287, 12288, 12289])
+@pytest.mark.parametrize("n", [2, 3, 511, 512, 513, 4898, 8193, 8194, 12287, 12288, 12289, 16384, 16385])
 @pytest.mark.parametrize("shape", ["random", "star", "deep", "binary"])
 def test_bit_exact(iso, oracle_lib, n, shape):
     from paper_1702_04739_gb300 import workloads
