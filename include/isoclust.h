@@ -103,12 +103,14 @@ typedef struct {
 
 /* spin_limit: the library's only device-side waits are the mbarrier waits
  * of the tensor-core Boruvka sweep (and of the omega screen, which reuses
- * it), between its copy, MMA and epilogue roles.  Each wait gives up after
- * spin_limit SM clock cycles: the kernel raises a timeout flag, lets the
- * copies and MMAs it already issued finish, frees its tensor memory and
- * returns; the call then returns ISOCLUST_ERR_TIMEOUT without walking the
- * unfinished tree, and the device stays usable.  A small value can make
- * calls fail on a healthy device.  Calls without the tensor-core sweep
+ * it) and of the omega kernel with the Gram on the tensor cores, between
+ * their copy, MMA and arithmetic roles.  Each wait gives up after
+ * spin_limit SM clock cycles (in the omega kernel, whose roles wait for one
+ * another's arithmetic, after at least 2e6 + 20,000 d): the kernel raises a
+ * timeout flag, lets the copies and MMAs it already issued finish, frees its
+ * tensor memory and returns; the call then returns ISOCLUST_ERR_TIMEOUT
+ * without walking the unfinished tree, and the device stays usable.  A small
+ * value can make calls fail on a healthy device.  Calls without these kernels
  * never wait (F64 input with a spin_limit takes none). */
 
 /* Test hook of the timeout path (no paper counterpart): while on (1), the

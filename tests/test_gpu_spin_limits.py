@@ -46,3 +46,14 @@ def test_any_limit_ends(iso, n, d, k):
     after = iso.cluster_detail(Xd, 3, 2.0)
     assert torch.equal(after["omega"], ref["omega"]) and torch.equal(after["parent"], ref["parent"])
     iso.set_omega_gram(-1)
+
+
+# the direct sums of long rows (two clusters far from one another) take some 10^7 cycles a block
+@pytest.mark.parametrize("n,d,sigma", [(3279, 1558, 40.0), (2000, 512, 23.0)])
+def test_limit_above_the_waits_for_hardware(iso, n, d, sigma):
+    Xd = torch.from_numpy(_points(n, d, 2)).cuda()
+    iso.set_omega_gram(1)
+    want = iso.cluster_detail(Xd, 2, sigma)
+    got = iso.cluster_detail(Xd, 2, sigma, iso.opts(spin_limit=1000000))
+    iso.set_omega_gram(-1)
+    assert torch.equal(got["omega"], want["omega"])
