@@ -474,10 +474,10 @@ int32_t isoclust_last_batched_graph_mode(void);
  * double-word sum.  Both keep d2 to about 2^-46 relative; omega agrees to
  * within the library's error bound, not bit for bit.
  * Tiles of 64 rows are centred on their centroid or on that of a near tile.
- * mode -1 (the default): the Gram on the tensor cores where tile pairs x
- * (d - 6) reach 65,536 and d 12 (20 for independent sets); 1: always (sets:
- * while its buffers stay within 16 GiB); 0: never.  Process-wide; other
- * values -> INVALID_ARG. */
+ * mode -1 (the default): the Gram on the tensor cores for a set's rows of 64
+ * dimensions or more, and where tile pairs x (d - 6) reach 65,536 and d 12 (20
+ * for independent sets); 1: always (sets: while its buffers stay within 16
+ * GiB); 0: never.  Process-wide; other values -> INVALID_ARG. */
 isoclust_status isoclust_set_omega_gram(int32_t mode);
 
 /* Pruned Boruvka rounds for one-set calls (Section 3.5's minimum spanning

@@ -30,22 +30,32 @@ size_t weights64_bytes(int64_t n, bool with_p);
 cudaError_t weights64_launch(const void *X, int64_t n, int32_t d, int dtype, double sigma, double alpha,
                              int include_self, double *omega, double *p, void *part, cudaStream_t s);
 constexpr size_t SYM_PART_LIMIT = size_t(16) << 30;   // symmetric sweep up to 16 GiB of partials
-// omega's Gram goes to the tensor cores by default when the tile pairs times
-// the dimensions (but for a few) outweigh its set-up (digit planes, block list:
-// some 80 us) and the one block per SM.  The omega stage in ms, CUDA cores /
-// Gram, by 64 x 64 tile pairs of the upper triangle (blobs):
-//      300 pairs: d = 64 .235/.310, 96 .286/.406
-//    1,128:       d = 48 .360/.395, 64 .410/.390
-//    4,465:       d = 16 .514/.555, 24 .596/.554, 64 1.04/.68
-//   12,403:       d = 8 .843/.941, 12 .957/.940, 32 1.51/.99
-//   49,141:       d = 8 2.77/2.63, 12 3.17/2.47, 64 9.1/2.9
+// omega's Gram goes to the tensor cores by default
+//  * for a set's rows of 64 dimensions or more, whatever it costs, because the
+//    sums of squares of k_weights_sym lose bits with every dimension (FP32 points
+//    near one another share a grid, and the low bits of squares on it are not
+//    even: the sums' roundings lean one way).  omega's error at sigma = 1 in
+//    1e-14, sums of squares / Gram (rms over rows against double-double sums,
+//    blobs): 1,000 x 64 2.8/.50, 2,000 x 130 11/.47, 800 x 620 97/1.6, 500 x
+//    1,558 232/7.4.  The stage in ms: 400 x 64 .178/.280, 2,000 x 130 .45/.70,
+//    800 x 620 .72/1.22, 500 x 1,558 1.6/4.9;
+//  * for shorter rows when the tile pairs times the dimensions (but for a few)
+//    outweigh its set-up (digit planes, block list: some 80 us) and the one
+//    block per SM.  The omega stage in ms, CUDA cores / Gram, by 64 x 64 tile
+//    pairs of the upper triangle (blobs):
+//      1,128:       d = 48 .360/.395
+//      4,465:       d = 16 .514/.555, 24 .596/.554
+//     12,403:       d = 8 .843/.941, 12 .957/.940, 32 1.51/.99
+//     49,141:       d = 8 2.77/2.63, 12 3.17/2.47
 // Independent sets have more half-empty blocks; 200 sets, 50,000 pairs:
 // d = 16 3.72/3.87, 24 4.05/3.48, 32 6.08/4.21; 32 sets, 250 pairs: 96 .155/.221.
 constexpr int64_t OMEGA_GRAM_MIN_WORK = 65536;        // tile pairs x (d - 6)
 constexpr int32_t OMEGA_GRAM_MIN_D = 12, OMEGA_GRAM_SETS_MIN_D = 20;
+constexpr int32_t OMEGA_GRAM_ALWAYS_D = 64;           // (one set)
 static bool omega_gram_pays(int64_t items, int32_t d, int32_t min_d) {
     return d >= min_d && items * (d - 6) >= OMEGA_GRAM_MIN_WORK;
 }
+
 size_t weights_sym_sets_bytes(int64_t n_pad, int64_t nitems, int32_t d);
 cudaError_t weights_launch_sym_sets(const float *Xp, int64_t n_pad, int32_t d, double sigma, int include_self,
                                     const unsigned long long *nnbits, double *omega, void *part, const int2 *witems,
@@ -487,7 +497,8 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     // eq. omega's Gram on the tensor cores (with the tensor-core screen)
     const int gram_mode = g_omega_gram.load(std::memory_order_relaxed);
     const bool gram = symmetric && use_tc &&
-                      (gram_mode == 1 || (gram_mode < 0 && omega_gram_pays(tri_items(n), d, OMEGA_GRAM_MIN_D)));
+                      (gram_mode == 1 || (gram_mode < 0 && (d >= OMEGA_GRAM_ALWAYS_D ||
+                                                           omega_gram_pays(tri_items(n), d, OMEGA_GRAM_MIN_D))));
     const bool weights64 = need_labels && dtype == ISOCLUST_F64 &&
                            (o.omega_mode == ISOCLUST_OMEGA_FULL || o.alpha != 0.0) &&
                            weights64_bytes(n, o.alpha != 0.0) <= SYM_PART_LIMIT;
