@@ -36,9 +36,9 @@ constexpr size_t SYM_PART_LIMIT = size_t(16) << 30;   // symmetric sweep up to 1
 //    near one another share a grid, and the low bits of squares on it are not
 //    even: the sums' roundings lean one way).  omega's error at sigma = 1 in
 //    1e-14, sums of squares / Gram (rms over rows against double-double sums,
-//    blobs): 1,000 x 64 2.8/.50, 2,000 x 130 11/.47, 800 x 620 97/1.6, 500 x
-//    1,558 232/7.4.  The stage in ms: 400 x 64 .178/.280, 2,000 x 130 .45/.70,
-//    800 x 620 .72/1.22, 500 x 1,558 1.6/4.9;
+//    blobs): 1,000 x 64 2.8/.43, 2,000 x 130 11/.43, 800 x 620 97/1.05, 500 x
+//    1,558 232/2.6.  The stage in ms: 400 x 64 .178/.286, 2,000 x 130 .45/.78,
+//    800 x 620 .72/1.34, 500 x 1,558 1.6/3.8;
 //  * for shorter rows when the tile pairs times the dimensions (but for a few)
 //    outweigh its set-up (digit planes, block list: some 80 us) and the one
 //    block per SM.  The omega stage in ms, CUDA cores / Gram, by 64 x 64 tile

@@ -39,3 +39,22 @@ def test_small_sets(iso, oracle_lib, n, d):
 def test_rule(iso, n, d, expect):
     iso.cluster_detail(torch.from_numpy(_blobs(n, d)).cuda(), 1, 1.0)
     assert iso.last_profile()["omega_symmetric"] == expect
+
+
+@pytest.mark.parametrize("n,d", [(64, 33), (64, 61), (64, 64), (50, 256), (64, 620), (33, 1300), (64, 1558)])
+def test_direct_sums_do_not_lean(iso, n, d):
+    """Pairs that cancel (clusters far from their tile's centre) take sums of squared differences.
+    Their roundings may not lean one way: the errors of omega's rows average out to less than 2^-50
+    of the exponent's half (d2 to y) and of the exponential and the sums (4 such units)."""
+    rng = np.random.default_rng(n + d)
+    X = (rng.uniform(-10, 10, size=(4, d))[np.arange(n) % 4] + rng.normal(size=(n, d))).astype(np.float32)
+    iso.set_omega_gram(1)
+    om = iso.cluster_detail(torch.from_numpy(X).cuda(), 1, 1.0)["omega"].cpu().numpy()
+    iso.set_omega_gram(-1)
+    assert iso.last_profile()["omega_gram_direct_pairs"] >= n * (n // 4 - 1)
+    L = X.astype(np.longdouble)
+    y = np.stack([np.sqrt(np.square(L - row).sum(1)) for row in L])
+    np.fill_diagonal(y, np.inf)
+    ref = np.exp(-y).sum(1)
+    err = ((om - ref) / ref).astype(np.float64)
+    assert abs(err.mean()) <= 2.0 ** -50 * (float(y.min(1).mean()) / 2 + 4.0), err.mean()
