@@ -557,7 +557,7 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     ISO_CUDA(check_finite(X, n * (int64_t)d, dtype, status, TC.f64 ? (unsigned long long *)(status + 2) : nullptr, s));
     // (words 4 to 7: the non-zeros)
     if (sp_look) ISO_CUDA(sparse_stats((const float *)X, n, d, status + 4, s));
-    struct { uint32_t st, pad; double absmax; unsigned long long nnz; uint32_t longest; float norm_max; } hv = {};
+    struct { uint32_t st, pad; double absmax; unsigned long long nnz; float norm_max; uint32_t pad2; } hv = {};
     ISO_CUDA(cudaMemcpyAsync(&hv, status, sizeof(hv), cudaMemcpyDeviceToHost, s));
     ISO_CUDA(cudaStreamSynchronize(s));
     if (hv.st) return map_status(hv.st, false);
@@ -595,7 +595,7 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     if (sp_mst) {
         tc_clear_last_variant();
         ISO_CUDA(sparse_build(SP, (const float *)X, s));
-        ISO_CUDA(mst_build_dist(M, TC, dmat, X, n, d, dtype, 0, status, s, &SP, (int32_t)hv.longest));
+        ISO_CUDA(mst_build_dist(M, TC, dmat, X, n, d, dtype, 0, status, s, &SP));
     } else if (dist_used) {
         tc_clear_last_variant();
         ISO_CUDA(mst_build_dist(M, TC, dmat, X, n, d, dtype, TC.scale_exp, status, s));

@@ -180,8 +180,7 @@ bool mst_dist_wanted(int64_t n, int32_t d, int dtype);
 bool mst_dist_sparse_wanted(int64_t n);
 struct SparseRows;
 cudaError_t mst_build_dist(MstScratch &S, TcScratch &T, float *D, const void *X, int64_t n, int32_t d, int dtype,
-                           int scale_exp, uint32_t *status, cudaStream_t s, const SparseRows *sp = nullptr,
-                           int32_t longest = 0);
+                           int scale_exp, uint32_t *status, cudaStream_t s, const SparseRows *sp = nullptr);
 // FP64 keys of the columns listed per row (T.nsurv, T.surv by point, T.permp
 // the identity) and of the rows listed for a rescan, into S.rowd2 / rowj
 cudaError_t tc_key_rows(TcScratch &T, MstScratch &S, const float *X, int64_t n, int32_t d, double mul, double add,

@@ -213,9 +213,15 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
     }
 }
 
-// The scan for rows as lists: the distances come from a Gram, within err (|x_i|^2
-// + |x_j|^2) of the true ones, so a column is a candidate when the smallest
-// distance its entry stands for is at most the smallest of the row's largest.
+// The scan for rows as lists: the distances come from a Gram, so a column is a
+// candidate when the smallest distance its entry stands for is at most the
+// smallest of the row's largest.  A product of rows takes a rounding per
+// dimension both hold, at most k = the entries of row i, of a partial sum below
+// |x_i| |x_j|, twice; the norms and the three last operations take one each of
+// |x_i|^2 + |x_j|^2 (v is at most twice that): within 2^-24 (2 k |x_i| |x_j| + 4
+// (|x_i|^2 + |x_j|^2)), and 10 % above.  (With the longest row's entries for
+// every pair and half the norms for the product, one full row of ones among
+// 50,000 of 41 entries had every column for a candidate: 29 ms -> 990.)
 // Keys from the lists (a dimension that neither row holds adds nothing to the
 // key), by a warp per candidate: the lanes find each entry's place in the two
 // lists' common order and leave its square there, one adds them up.  (One
@@ -224,10 +230,10 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
 // columns hold two candidates or more looks at them again.
 constexpr int SC_THREADS = 512, SC_CAND = 128, SC_LIST = 128;
 __global__ void __launch_bounds__(SC_THREADS) k_sparse_scan(const SparseRows R, int64_t n, const float *__restrict__ D,
-                                                            int64_t ld, float err, float add,
+                                                            int64_t ld, float add,
                                                             const int32_t *__restrict__ comp, double *__restrict__ rowd2,
                                                             int32_t *__restrict__ rowj,
-                                                            unsigned long long *__restrict__ cd2, const int32_t *counters) {
+                                                            unsigned long long *__restrict__ cd2, int32_t *counters) {
     if (!dist_active(counters)) return;
     constexpr int NW = SC_THREADS / 32;
     __shared__ float smin[NW];
@@ -241,20 +247,22 @@ __global__ void __launch_bounds__(SC_THREADS) k_sparse_scan(const SparseRows R, 
     const int64_t i = blockIdx.x;
     const int32_t ci = comp[i];
     const float *row = D + i * ld;
-    const float ni = R.norm1[i];
+    const float ri = R.root[i];
     const int32_t a0 = R.rowptr[i], alen = R.rowptr[i + 1] - a0;
+    constexpr float U = 1.1f * 5.9604645e-08f;
+    const float gk = __fmul_ru(__fmul_ru(2.0f * U, (float)(alen + 1)), ri), gn = 5.0f * U, own = __fmul_ru(gn, __fmul_ru(ri, ri));
     for (int e = tid; e < alen && e < SC_LIST; e += SC_THREADS) {
         ac[e] = R.rcol[a0 + e];
         av[e] = R.rval[a0 + e];
     }
     if (tid == 0) scnt = 0;
     const int64_t n4 = n & ~(int64_t)3;
-    auto wide = [&](float nj) { return __fmul_ru(err, __fadd_ru(ni, nj)); };
+    auto wide = [&](float rj) { return __fmaf_ru(rj, __fmaf_ru(gn, rj, gk), own); };
     // the thread's two smallest, and the column of the smaller
     float m = INFINITY, low = INFINITY, low2 = INFINITY;
     int32_t lowj = -1;
-    auto first = [&](float v, float nj, int64_t j) {
-        const float w = wide(nj), l = __fsub_rd(v, w);
+    auto first = [&](float v, float rj, int64_t j) {
+        const float w = wide(rj), l = __fsub_rd(v, w);
         m = fminf(m, __fadd_ru(v, w));
         low2 = fminf(low2, fmaxf(low, l));
         if (l < low) {
@@ -266,13 +274,13 @@ __global__ void __launch_bounds__(SC_THREADS) k_sparse_scan(const SparseRows R, 
     for (int64_t j = 4 * tid; j < n4; j += 4 * SC_THREADS) {
         const float4 v = *reinterpret_cast<const float4 *>(row + j);
         const int4 c = *reinterpret_cast<const int4 *>(comp + j);
-        const float4 q = *reinterpret_cast<const float4 *>(R.norm1 + j);
+        const float4 q = *reinterpret_cast<const float4 *>(R.root + j);
         if (c.x != ci) first(v.x, q.x, j);
         if (c.y != ci) first(v.y, q.y, j + 1);
         if (c.z != ci) first(v.z, q.z, j + 2);
         if (c.w != ci) first(v.w, q.w, j + 3);
     }
-    if (n4 + tid < n && comp[n4 + tid] != ci) first(row[n4 + tid], R.norm1[n4 + tid], n4 + tid);
+    if (n4 + tid < n && comp[n4 + tid] != ci) first(row[n4 + tid], R.root[n4 + tid], n4 + tid);
     for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) smin[wp] = m;
     __syncthreads();
@@ -316,8 +324,8 @@ __global__ void __launch_bounds__(SC_THREADS) k_sparse_scan(const SparseRows R, 
             take(key(R.rcol + a0, R.rval + a0, alen, R.rcol + b0, R.rval + b0, R.rowptr[j + 1] - b0), (int32_t)j);
         }
     };
-    auto again = [&](float v, float nj, int32_t c, int64_t j) {
-        if (c != ci && __fsub_rd(v, wide(nj)) <= thr) see(j);
+    auto again = [&](float v, float rj, int32_t c, int64_t j) {
+        if (c != ci && __fsub_rd(v, wide(rj)) <= thr) see(j);
     };
     if (low <= thr && low2 > thr) {
         see(lowj);
@@ -325,16 +333,17 @@ __global__ void __launch_bounds__(SC_THREADS) k_sparse_scan(const SparseRows R, 
         for (int64_t j = 4 * tid; j < n4; j += 4 * SC_THREADS) {
             const float4 v = *reinterpret_cast<const float4 *>(row + j);
             const int4 c = *reinterpret_cast<const int4 *>(comp + j);
-            const float4 q = *reinterpret_cast<const float4 *>(R.norm1 + j);
+            const float4 q = *reinterpret_cast<const float4 *>(R.root + j);
             again(v.x, q.x, c.x, j);
             again(v.y, q.y, c.y, j + 1);
             again(v.z, q.z, c.z, j + 2);
             again(v.w, q.w, c.w, j + 3);
         }
-        if (n4 + tid < n) again(row[n4 + tid], R.norm1[n4 + tid], comp[n4 + tid], n4 + tid);
+        if (n4 + tid < n) again(row[n4 + tid], R.root[n4 + tid], comp[n4 + tid], n4 + tid);
     }
     __syncthreads();
     const int nc = scnt < SC_CAND ? scnt : SC_CAND;
+    if (tid == 0 && scnt > SC_CAND) atomicAdd(counters + MC_OVERFLOW, 1);      // (the call's count of such rows)
     for (int q = wp; q < nc; q += NW) {
         const int32_t j = scand[q], b0 = R.rowptr[j], blen = R.rowptr[j + 1] - b0;
         const bool fits = alen <= SC_LIST && blen <= SC_LIST;
@@ -533,7 +542,7 @@ bool mst_dist_wanted(int64_t n, int32_t d, int dtype) {
 }
 
 cudaError_t mst_build_dist(MstScratch &S, TcScratch &T, float *D, const void *X, int64_t n, int32_t d, int dtype,
-                           int scale_exp, uint32_t *status, cudaStream_t s, const SparseRows *sp, int32_t longest) {
+                           int scale_exp, uint32_t *status, cudaStream_t s, const SparseRows *sp) {
     const int64_t Tn = ceil_div(n, DS_T), ld = Tn * DS_T;
     const unsigned tiles = (unsigned)(Tn * (Tn + 1) / 2);
     const bool f64 = dtype == ISOCLUST_F64, inl = sp || f64 || d <= MST_DIST_INLINE_MAX_D;
@@ -552,10 +561,6 @@ cudaError_t mst_build_dist(MstScratch &S, TcScratch &T, float *D, const void *X,
     const double u = 5.9604644775390625e-08, er = 1.1 * (double)(d + 3) * u;
     const double mul = (1.0 + er) / (1.0 - er), add = (double)(d + 1) * 1.401298464324817e-45 * 4.0;
     const float mul32 = (float)(mul * (1.0 + 1e-6)), add32 = (float)(2.01 * add) + 1.401298464324817e-45f;
-    // A Gram's distance: the products' sums (a rounding per entry of the shorter
-    // row, 2^-24 of |x_i| |x_j| <= (|x_i|^2 + |x_j|^2) / 2 each, twice), the norms
-    // and the two last operations: within (longest + 5) 2^-24 (|x_i|^2 + |x_j|^2)
-    const float err = sp ? (float)(1.1 * (double)(longest + 6) * u) : 0.0f;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if ((e = cudaStreamIsCapturing(s, &cs))) return e;
     const bool ask = cs == cudaStreamCaptureStatusNone;
@@ -567,7 +572,7 @@ cudaError_t mst_build_dist(MstScratch &S, TcScratch &T, float *D, const void *X,
                                                                     S.rowd2, S.rowj, S.cd2, T.nsurv, T.surv,           \
                                                                     S.ovf_rows, S.counters)
         if (sp) {
-            k_sparse_scan<<<(unsigned)n, SC_THREADS, 0, ISO_S(s)>>>(*sp, n, D, ld, err, add32, S.comp, S.rowd2, S.rowj, S.cd2,
+            k_sparse_scan<<<(unsigned)n, SC_THREADS, 0, ISO_S(s)>>>(*sp, n, D, ld, add32, S.comp, S.rowd2, S.rowj, S.cd2,
                                                                    S.counters);
         } else if (f64) {
             ISO_SCAN(double, true);

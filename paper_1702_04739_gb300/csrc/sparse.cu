@@ -20,7 +20,6 @@ __global__ void __launch_bounds__(256) k_sp_stats(const float *__restrict__ X, i
                                                   uint32_t *__restrict__ stat) {
     const int lane = threadIdx.x & 31;
     unsigned long long total = 0;
-    unsigned longest = 0;
     float nmax = 0.0f;
     const int64_t gs = (int64_t)gridDim.x * 8;
     for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < n; r += gs) {
@@ -36,19 +35,18 @@ __global__ void __launch_bounds__(256) k_sp_stats(const float *__restrict__ X, i
             q += __shfl_xor_sync(0xffffffffu, q, o);
         }
         total += c;
-        longest = max(longest, c);
         nmax = fmaxf(nmax, q);
     }
     if (lane == 0) {
         atomicAdd(reinterpret_cast<unsigned long long *>(stat), total);
-        atomicMax(stat + 2, longest);
-        atomicMax(stat + 3, __float_as_uint(nmax));          // (non-negative floats: their bits are in order)
+        atomicMax(stat + 2, __float_as_uint(nmax));          // (non-negative floats: their bits are in order)
     }
 }
 
-// one warp per padded row: its non-zeros, |x|^2 (FP64 sum) as a double-word
+// one warp per padded row: its non-zeros, |x|^2 (FP64 sum) as a double-word, |x|
+// rounded up
 __global__ void __launch_bounds__(256) k_sp_count(const float *__restrict__ X, int64_t n, int64_t n_pad, int32_t d,
-                                                  int32_t *__restrict__ cnt, float2 *__restrict__ norm, float *__restrict__ norm1) {
+                                                  int32_t *__restrict__ cnt, float2 *__restrict__ norm, float *__restrict__ root) {
     const int lane = threadIdx.x & 31;
     const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (r > n_pad) return;
@@ -69,7 +67,7 @@ __global__ void __launch_bounds__(256) k_sp_count(const float *__restrict__ X, i
         if (r < n_pad) {
             const float h = (float)q;
             norm[r] = make_float2(h, (float)(q - (double)h));
-            norm1[r] = h;
+            root[r] = __double2float_ru(sqrt(q));
         }
     }
 }
@@ -186,7 +184,7 @@ void SparseRows::carve(Arena &A, int64_t n_, int32_t d_, int64_t nnz) {
     goff = A.take<uint32_t>((size_t)(n_pad / 32) * d);
     gent = A.take<float2>(nnz);
     norm = A.take<float2>(n_pad);
-    norm1 = A.take<float>(n_pad);
+    root = A.take<float>(n_pad);
     // rows up to twice the average length and a little wholly in slots
     width = (int32_t)(2 * ceil_div(nnz, n) + 8);
     ell = A.take<float2>((size_t)n_pad * width);
@@ -208,7 +206,7 @@ bool sparse_pays(int64_t n, int32_t d, int64_t nnz, float norm_max) {
 
 cudaError_t sparse_build(SparseRows &R, const float *X, cudaStream_t s) {
     cudaError_t e;
-    k_sp_count<<<(unsigned)ceil_div(R.n_pad + 1, 8), 256, 0, ISO_S(s)>>>(X, R.n, R.n_pad, R.d, R.cnt, R.norm, R.norm1);
+    k_sp_count<<<(unsigned)ceil_div(R.n_pad + 1, 8), 256, 0, ISO_S(s)>>>(X, R.n, R.n_pad, R.d, R.cnt, R.norm, R.root);
     if ((e = exclusive_scan_i32(R.cnt, R.rowptr, R.n_pad + 1, R.tmp, s))) return e;
     k_sp_rows<<<(unsigned)ceil_div(R.n, 8), 256, 0, ISO_S(s)>>>(X, R.n, R.d, R.rowptr, R.cap, R.rcol, R.rval, R.width, R.ell);
     static std::atomic<unsigned long long> seen{0};

@@ -21,7 +21,7 @@ struct SparseRows {
     uint32_t *goff = nullptr;
     float2 *gent = nullptr;
     float2 *norm = nullptr;            // |x|^2 as a double-word
-    float *norm1 = nullptr;            // its leading word
+    float *root = nullptr;             // |x|, rounded up
     int32_t width = 0;
     float2 *ell = nullptr;             // [n_pad / 32][width][32]
 
@@ -31,8 +31,8 @@ struct SparseRows {
     void carve(Arena &A, int64_t n, int32_t d, int64_t nnz);
 };
 
-// Non-zeros, the longest row and the largest |x|^2 of the rows of X into
-// stat[0..1] (64 bits), [2] and [3] (FP32 bits), zeroed before.
+// Non-zeros and the largest |x|^2 of the rows of X into stat[0..1] (64 bits)
+// and [2] (FP32 bits), zeroed before.
 cudaError_t sparse_stats(const float *X, int64_t n, int32_t d, uint32_t *stat, cudaStream_t s);
 // Whether rows of that many non-zeros take the sparse kernels.
 bool sparse_pays(int64_t n, int32_t d, int64_t nnz, float norm_max);
