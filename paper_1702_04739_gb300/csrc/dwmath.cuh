@@ -40,6 +40,14 @@ __device__ __forceinline__ void dw_add(float &h, float &l, float bh, float bl) {
     fast_two_sum(s, e, h, l);
 }
 
+// (a - b)^2 as a double-word.  A difference's rounding error enters with its
+// square too: without it every squared difference is 2^-50 too small on average.
+__device__ __forceinline__ void dw_square_diff(float a, float b, float &p, float &q) {
+    float s, e;
+    two_sum(a, -b, s, e);
+    p = __fmul_rn(s, s);
+    q = __fmaf_rn(e, e, __fmaf_rn(__fadd_rn(s, s), e, __fmaf_rn(s, s, -p)));
+}
 
 // exp(-z) * 1 for z given as a double-word, result as a double-word.
 __device__ __forceinline__ void dw_exp_neg(float zh, float zl, const float2 *__restrict__ tab, float &oh, float &ol) {

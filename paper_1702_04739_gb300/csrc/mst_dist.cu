@@ -219,7 +219,8 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
 // dimension both hold, at most k = the entries of row i, of a partial sum below
 // |x_i| |x_j|, twice; the norms and the three last operations take one each of
 // |x_i|^2 + |x_j|^2 (v is at most twice that): within 2^-24 (2 k |x_i| |x_j| + 4
-// (|x_i|^2 + |x_j|^2)), and 10 % above.  (With the longest row's entries for
+// (|x_i|^2 + |x_j|^2)), and 10 % above; an entry with its sign set is a direct
+// sum, within one rounding of itself.  (With the longest row's entries for
 // every pair and half the norms for the product, one full row of ones among
 // 50,000 of 41 entries had every column for a candidate: 29 ms -> 990.)
 // Keys from the lists (a dimension that neither row holds adds nothing to the
@@ -261,8 +262,9 @@ __global__ void __launch_bounds__(SC_THREADS) k_sparse_scan(const SparseRows R, 
     // the thread's two smallest, and the column of the smaller
     float m = INFINITY, low = INFINITY, low2 = INFINITY;
     int32_t lowj = -1;
-    auto first = [&](float v, float rj, int64_t j) {
-        const float w = wide(rj), l = __fsub_rd(v, w);
+    auto margin = [&](float v, float rj) { return __float_as_int(v) < 0 ? __fmul_ru(-2.0f * U, v) : wide(rj); };
+    auto first = [&](float v, float w, int64_t j) {
+        const float l = __fsub_rd(v, w);
         m = fminf(m, __fadd_ru(v, w));
         low2 = fminf(low2, fmaxf(low, l));
         if (l < low) {
@@ -275,12 +277,20 @@ __global__ void __launch_bounds__(SC_THREADS) k_sparse_scan(const SparseRows R, 
         const float4 v = *reinterpret_cast<const float4 *>(row + j);
         const int4 c = *reinterpret_cast<const int4 *>(comp + j);
         const float4 q = *reinterpret_cast<const float4 *>(R.root + j);
-        if (c.x != ci) first(v.x, q.x, j);
-        if (c.y != ci) first(v.y, q.y, j + 1);
-        if (c.z != ci) first(v.z, q.z, j + 2);
-        if (c.w != ci) first(v.w, q.w, j + 3);
+        if ((__float_as_int(v.x) | __float_as_int(v.y) | __float_as_int(v.z) | __float_as_int(v.w)) >= 0) {
+            if (c.x != ci) first(v.x, wide(q.x), j);
+            if (c.y != ci) first(v.y, wide(q.y), j + 1);
+            if (c.z != ci) first(v.z, wide(q.z), j + 2);
+            if (c.w != ci) first(v.w, wide(q.w), j + 3);
+        } else {                               // (a direct sum among them)
+            if (c.x != ci) first(fabsf(v.x), margin(v.x, q.x), j);
+            if (c.y != ci) first(fabsf(v.y), margin(v.y, q.y), j + 1);
+            if (c.z != ci) first(fabsf(v.z), margin(v.z, q.z), j + 2);
+            if (c.w != ci) first(fabsf(v.w), margin(v.w, q.w), j + 3);
+        }
     }
-    if (n4 + tid < n && comp[n4 + tid] != ci) first(row[n4 + tid], R.root[n4 + tid], n4 + tid);
+    if (n4 + tid < n && comp[n4 + tid] != ci)
+        first(fabsf(row[n4 + tid]), margin(row[n4 + tid], R.root[n4 + tid]), n4 + tid);
     for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) smin[wp] = m;
     __syncthreads();
@@ -325,7 +335,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_sparse_scan(const SparseRows R, 
         }
     };
     auto again = [&](float v, float rj, int32_t c, int64_t j) {
-        if (c != ci && __fsub_rd(v, wide(rj)) <= thr) see(j);
+        if (c != ci && __fsub_rd(fabsf(v), margin(v, rj)) <= thr) see(j);
     };
     if (low <= thr && low2 > thr) {
         see(lowj);

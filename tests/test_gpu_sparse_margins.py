@@ -1,6 +1,6 @@
 """The spanning tree from rows as lists: the margin of a row's candidates
-follows from its own entries and norms, so that one full or long row does not
-make candidates of every column; and rows with more candidates than a block
+follows from its own entries and norms, so that neither one full or long row nor
+rows far from the origin make candidates of every column; and rows with more candidates than a block
 keys together (exact ties) give the oracle's tree all the same."""
 import numpy as np
 import pytest
@@ -40,6 +40,18 @@ def test_one_full_row(iso, oracle_lib, row):
     X = _unit_rows(n, d, 41, rng)
     X[77] = {"ones": np.ones(d), "random": rng.normal(size=d) / 64.0, "long": 300.0 * X[77]}[row]
     assert _same_tree(iso, oracle_lib, X) == 0          # no row with more than 128 candidates
+
+
+@pytest.mark.parametrize("value", [30.0, 1000.0, -3e6])
+@pytest.mark.parametrize("rows", ["all", "half", "one block"])
+def test_far_from_the_origin(iso, oracle_lib, value, rows):
+    n, d = 900, 1024
+    X = _unit_rows(n, d, 20, np.random.default_rng(5))
+    X[{"all": slice(None), "half": slice(None, None, 2), "one block": slice(100, 300)}[rows], 5] = value
+    X[201] = X[200]
+    # products that cancel make no candidates of every column; of two groups that far apart the one
+    # round that joins them finds the distances between them tied in FP32
+    assert _same_tree(iso, oracle_lib, X) <= (0 if rows == "all" else n)
 
 
 @pytest.mark.parametrize("kind", ["one-hot", "equal", "identical"])
