@@ -17,8 +17,14 @@
  *     stream).  All work is queued on it; every call synchronises `stream`
  *     once before it returns so that the status it returns is final.
  *   - Internal scratch memory is allocated by the library on the current
- *     device, cached per device and reused by later calls (grow-only).  Calls
- *     on the same device from several host threads are serialised.
+ *     device, cached per device and reused by later calls (grow-only, with up
+ *     to 1 GiB to spare).  Its largest parts are there for speed, and a call
+ *     that finds no room for them does without: the n x n FP32 distances of a
+ *     set of rows with few non-zeros (up to 17 GB at 65,536 points), the pair
+ *     sums' partials of FP64 input (up to 16 GiB), the digit planes of omega's
+ *     Gram for rows under 64 dimensions and for independent sets (22 bytes per
+ *     value, for sets up to 16 GiB).  Calls on the same device from several
+ *     host threads are serialised.
  *   - No call throws.  On a non-OK status the outputs are unspecified and
  *     isoclust_last_error() holds a one-line reason (per host thread).
  *   - Indices are 0-based.  n is limited to 2^31 - 2 points.

@@ -164,7 +164,8 @@ void *scratch_acquire(size_t bytes, cudaStream_t stream, isoclust_status *st) {
         g_scratch[dev] = nullptr;
         g_scratch_cap[dev] = 0;
     }
-    size_t want = bytes + bytes / 4 + (1u << 20);
+    // (room to grow, but no more than 1 GiB kept from the caller's own tensors)
+    size_t want = bytes + (bytes / 4 < (size_t(1) << 30) ? bytes / 4 : size_t(1) << 30) + (1u << 20);
     void *p = nullptr;
     cudaError_t e = cudaMalloc(&p, want);
     if (e != cudaSuccess) {
@@ -443,12 +444,12 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     // waits (such a call cannot run out of it).
     TC.f64 = dtype == ISOCLUST_F64 && o.precision == ISOCLUST_PREC_AUTO && o.spin_limit == 0 && !TC.stall_test &&
              tc_supported();
-    const bool tc_any = use_tc || TC.f64;
+    bool tc_any = use_tc || TC.f64;
     // a small set's rounds on stored distances; whoever asks for the
     // tensor-core sweep (precision, variant, pruning, a limit on its waits)
     // gets it
-    const bool dist = tc_any && !sh && o.precision == ISOCLUST_PREC_AUTO && o.spin_limit == 0 && !TC.stall_test &&
-                      tc_forced_variant() < 0 && prune_mode() != 1 && mst_dist_wanted(n, d, dtype);
+    bool dist = tc_any && !sh && o.precision == ISOCLUST_PREC_AUTO && o.spin_limit == 0 && !TC.stall_test &&
+                tc_forced_variant() < 0 && prune_mode() != 1 && mst_dist_wanted(n, d, dtype);
     float *dmat = nullptr;
     // rows with few non-zeros, known once the points are looked at: room is
     // asked for only then
@@ -496,12 +497,12 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
                            weights_sym_bytes(n, d) <= SYM_PART_LIMIT;
     // eq. omega's Gram on the tensor cores (with the tensor-core screen)
     const int gram_mode = g_omega_gram.load(std::memory_order_relaxed);
-    const bool gram = symmetric && use_tc &&
-                      (gram_mode == 1 || (gram_mode < 0 && (d >= OMEGA_GRAM_ALWAYS_D ||
-                                                           omega_gram_pays(tri_items(n), d, OMEGA_GRAM_MIN_D))));
-    const bool weights64 = need_labels && dtype == ISOCLUST_F64 &&
-                           (o.omega_mode == ISOCLUST_OMEGA_FULL || o.alpha != 0.0) &&
-                           weights64_bytes(n, o.alpha != 0.0) <= SYM_PART_LIMIT;
+    bool gram = symmetric && use_tc &&
+                (gram_mode == 1 || (gram_mode < 0 && (d >= OMEGA_GRAM_ALWAYS_D ||
+                                                     omega_gram_pays(tri_items(n), d, OMEGA_GRAM_MIN_D))));
+    bool weights64 = need_labels && dtype == ISOCLUST_F64 &&
+                     (o.omega_mode == ISOCLUST_OMEGA_FULL || o.alpha != 0.0) &&
+                     weights64_bytes(n, o.alpha != 0.0) <= SYM_PART_LIMIT;
     auto carve = [&](Arena &A, MstScratch &M, TreeScratch &TS, double **phi, double **om, double **pp, double **omtmp,
                      uint32_t **status) {
         *status = A.take<uint32_t>(8);
@@ -541,7 +542,18 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     Arena meas;
     carve(meas, M, TS, &phi, &om, &pp, &omtmp, &status);
     void *base = scratch_acquire(meas.off, s, &st);
-    if (!base) return st;
+    if (!base) {
+        // no room: without what is there for speed alone (FP64 input: the
+        // sweep's copy and the pair sums' partials, up to 16 GiB of them; FP32:
+        // the distance matrix, the digit planes of short rows)
+        TC.f64 = dist = weights64 = false;
+        tc_any = use_tc;
+        if (gram_mode < 0 && d < OMEGA_GRAM_ALWAYS_D) gram = false;
+        meas = Arena();
+        carve(meas, M, TS, &phi, &om, &pp, &omtmp, &status);
+        base = scratch_acquire(meas.off, s, &st);
+        if (!base) return st;
+    }
     Arena A{(char *)base, meas.off + 4096, 0, false};
     carve(A, M, TS, &phi, &om, &pp, &omtmp, &status);
     if (A.overflow) return fail(ISOCLUST_ERR_INTERNAL, "scratch carve overflow");
@@ -911,8 +923,8 @@ static isoclust_status cluster_sets_impl(const void *X, const int64_t *offsets, 
     } B;
     const int gram_mode = g_omega_gram.load(std::memory_order_relaxed);
     // (many sets: within the same limit as the partials of one)
-    const bool gram = nitems > 0 && omega_tc_bytes(n_pad64, d, nitems) <= SYM_PART_LIMIT &&
-                      (gram_mode == 1 || (gram_mode < 0 && omega_gram_pays(nitems, d, OMEGA_GRAM_SETS_MIN_D)));
+    bool gram = nitems > 0 && omega_tc_bytes(n_pad64, d, nitems) <= SYM_PART_LIMIT &&
+                (gram_mode == 1 || (gram_mode < 0 && omega_gram_pays(nitems, d, OMEGA_GRAM_SETS_MIN_D)));
     auto carve = [&](Arena &A) {
         B.status = A.take<uint32_t>(4);
         B.plan = A.take<int64_t>(plan.size());
@@ -943,6 +955,13 @@ static isoclust_status cluster_sets_impl(const void *X, const int64_t *offsets, 
     Arena meas;
     carve(meas);
     void *base = scratch_acquire(meas.off, s, &st);
+    if (!base && gram && gram_mode < 0) {
+        // no room for the digit planes: the sums of squares
+        gram = false;
+        meas = Arena();
+        carve(meas);
+        base = scratch_acquire(meas.off, s, &st);
+    }
     if (!base) return st;
     Arena A{(char *)base, meas.off + 4096, 0, false};
     carve(A);
@@ -1347,7 +1366,7 @@ isoclust_status isoclust_vertex_weights(const void *X, int64_t n, int32_t d, int
     TC.stall_test = g_stall_test.load(std::memory_order_relaxed);
     const int tsplits = use_tc ? tc_splits(n) : 1;
     const size_t w64 = fp64 ? weights64_bytes(n, o.alpha != 0.0 && p) : 0;
-    const bool sym64 = fp64 && w64 <= SYM_PART_LIMIT;
+    bool sym64 = fp64 && w64 <= SYM_PART_LIMIT;
     void *part64 = nullptr;
     const int dev = current_device();
     std::lock_guard<std::mutex> lock(g_call_mu[dev]);
@@ -1357,8 +1376,15 @@ isoclust_status isoclust_vertex_weights(const void *X, int64_t n, int32_t d, int
     status = meas.take<uint32_t>(4);
     M.carve(meas, n, splits);
     if (use_tc) TC.carve(meas, n, d, tsplits);
+    const size_t without = meas.off;
     if (sym64) meas.take<unsigned char>(w64);
     void *base = scratch_acquire(meas.off, s, &st);
+    if (!base && sym64) {
+        // no room for the pair sums' partials: a thread per row
+        sym64 = false;
+        meas.off = without;
+        base = scratch_acquire(meas.off, s, &st);
+    }
     if (!base) return st;
     Arena A{(char *)base, meas.off + 4096, 0, false};
     status = A.take<uint32_t>(4);
