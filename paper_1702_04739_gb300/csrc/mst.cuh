@@ -36,6 +36,8 @@ struct MstScratch {
 
 int mst_splits(int64_t n);
 
+constexpr int TC_SURV = 8;              // FP64-keyed columns per row (more: rescan)
+
 // Tensor-core sweep state (mst_tc.cu): centred BF16 hi/lo copies of X in a
 // padded row space of 128-row tiles, their TMA maps, squared norms and the
 // best-8 candidate lists of every (list, row).  One set: rows in norm order,
@@ -60,7 +62,7 @@ struct TcScratch {
     uint64_t *keys = nullptr, *kbuf = nullptr;
     float *tv = nullptr, *tu = nullptr;            // per (list, row): best-8 candidate-block lower bounds, best upper bound
     int32_t *tj = nullptr;
-    int32_t *nsurv = nullptr, *surv = nullptr;     // per row: columns to key in FP64 (padded column indices)
+    int32_t *nsurv = nullptr, *surv = nullptr;     // per row: columns to key in FP64 (padded column indices, TC_SURV a row)
     unsigned int *rmin = nullptr;                  // per row: FP32 minimum of a rescan (bits)
     uint32_t *err = nullptr;
     uint32_t *qctr = nullptr;                      // the sweep's work-item counter (zeroed before each launch)

@@ -110,9 +110,9 @@ __global__ void __launch_bounds__(256) k_dist_tiles(const P *__restrict__ X, int
 
 // One row per block.  INLINE (short rows): a thread keys its own columns, the
 // block's best goes to rowd2 / rowj and to its component's minimum.  Else the
-// columns go to surv for the FP64 keys of long rows, more than SURV of them
+// columns go to surv for the FP64 keys of long rows, more than TC_SURV of them
 // (exact ties) to the rescan.
-constexpr int DSC_THREADS = 128, DSC_SURV = 8;
+constexpr int DSC_THREADS = 128;
 template <class P, bool INLINE>
 __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__ X, int64_t n, int32_t d,
                                                            const float *__restrict__ D, int64_t ld, float mul, float add,
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
             }
         } else {
             const int q = atomicAdd(&scnt, 1);
-            if (q < DSC_SURV) surv[i * DSC_SURV + q] = (int32_t)j;
+            if (q < TC_SURV) surv[i * TC_SURV + q] = (int32_t)j;
         }
     };
     if (low <= thr)
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(DSC_THREADS) k_dist_scan(const P *__restrict__
         if (tid == 0) {
             nsurv[i] = scnt;
             rowj[i] = -1;
-            if (scnt > DSC_SURV) {
+            if (scnt > TC_SURV) {
                 ovf[atomicAdd(counters + MC_OVERFLOW, 1)] = (int32_t)i;
                 rowj[i] = -2;
             }

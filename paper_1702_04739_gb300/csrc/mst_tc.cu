@@ -52,7 +52,6 @@ constexpr int TC_TOPK = 8;                                // best candidate bloc
 // Columns per candidate block: 64 (one set, d_pad <= 64: the epilogue is
 // the sweep's limit) or 32 (independent sets or wider rows: the recheck's
 // column reads are the limit).
-constexpr int TC_SURV = 8;                                // FP64-keyed columns per row (more: rescan)
 constexpr int TC_QD = 4;                                  // work-item queue slots (producer -> MMA, epilogue)
 constexpr long long TC_WAIT_CYCLES = 4000000000LL;         // default bound of one wait (about 2 s)
 
