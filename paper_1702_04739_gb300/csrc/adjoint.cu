@@ -698,13 +698,13 @@ cudaError_t adjoint_launch(const void *X, int32_t dtype, int64_t n, int32_t d, c
     static const ExpTable tab = make_exp_table();
     const unsigned gp = (unsigned)(nit < num_sms() ? (nit > 0 ? nit : 1) : num_sms());
     const unsigned gr = grid_for((na + nb) * d);
-    static bool attr = false;
-    if (!attr) {
+    static std::atomic<unsigned long long> seen{0};
+    if (first_on_device(seen)) {
         if ((e = cudaFuncSetAttribute(k_pair_grad<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm)))
             return e;
         if ((e = cudaFuncSetAttribute(k_pair_grad<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm)))
             return e;
-        attr = true;
+        done_on_device(seen);
     }
     if (dtype == ISOCLUST_F64) {
         const double *Xd = (const double *)X;

@@ -1633,8 +1633,8 @@ cudaError_t tc_prepare(TcScratch &T, const float *X, int64_t n, int32_t d, cudaS
     if ((e = cudaMemsetAsync(T.err, 0, sizeof(uint32_t), s))) return e;
     if ((e = make_map(&T.map_h, T.xh, T.n_pad, T.d_pad))) return e;
     if ((e = make_map(&T.map_l, T.xl, T.n_pad, T.d_pad))) return e;
-    static bool attr = false;
-    if (!attr) {
+    static std::atomic<unsigned long long> seen{0};
+    if (first_on_device(seen)) {
 #define ISO_SMEM_ATTR(AKV, SCR, CWV)                                                                              \
     if ((e = cudaFuncSetAttribute(k_sweep_tc<AKV, SCR, CWV>, cudaFuncAttributeMaxDynamicSharedMemorySize,         \
                                   tc_smem(AKV))))                                                                 \
@@ -1649,7 +1649,7 @@ cudaError_t tc_prepare(TcScratch &T, const float *X, int64_t n, int32_t d, cudaS
         ISO_SMEM_ATTR(1, true, 64)
         ISO_SMEM_ATTR(2, true, 64)
 #undef ISO_SMEM_ATTR
-        attr = true;
+        done_on_device(seen);
     }
     return cudaGetLastError();
 }
