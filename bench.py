@@ -254,8 +254,7 @@ def omega_fused_roofline(prof, peaks, src, alu_peak, sms, kernel_ms, items, d, a
     blocks, direct = prof[-1]["omega_gram_blocks"], prof[-1].get("omega_gram_direct_pairs", 0)
     seconds = kernel_ms / 1000.0
     bf16 = peaks.get("bf16_tflops", 1900.0)
-    # rows with few non-zeros (long rows whose tree took no tensor-core sweep): the Gram from their lists, no MMAs
-    lists = d >= 512 and not prof[-1].get("mst_tiles_full", 1)
+    lists = prof[-1].get("omega_path") == "gram_lists"       # rows with few non-zeros: no MMAs
     tc = 0.0 if lists else blocks * 34 * 2.0 * 128 * 64 * (-(-d // 16) * 16) / seconds / 1e12
     alu = (items * 4096.0 * 147.0 + direct * (18.75 * d + 95.0)) / seconds / 1e12
     alg = alg_flop / seconds / 1e12

@@ -461,6 +461,20 @@ isoclust_status isoclust_set_sweep_variant(int32_t variant);
  * thread (0..3), or -1 when none ran (FP32/FP64 sweep, stored distances). */
 int32_t isoclust_last_sweep_variant(void);
 
+/* What the last isoclust_cluster* call on this host thread that returned OK
+ * used: paths2[0] for the spanning tree, paths2[1] for omega. */
+enum {
+    ISOCLUST_PATH_TREE_SWEEP = 0,      /* the FP64 sweep, or FP32 candidates and FP64 keys */
+    ISOCLUST_PATH_TREE_TC_SWEEP = 1,   /* the tensor-core sweep                            */
+    ISOCLUST_PATH_TREE_STORED = 2,     /* all distances stored, rows in full (small sets)  */
+    ISOCLUST_PATH_TREE_LISTS = 3,      /* all distances stored, rows by their non-zeros    */
+    ISOCLUST_PATH_OMEGA_NONE = 0,      /* the tree alone, or omega from the tree's edges   */
+    ISOCLUST_PATH_OMEGA_SUMS = 1,      /* sums of squared differences                      */
+    ISOCLUST_PATH_OMEGA_GRAM_TC = 2,   /* the Gram on the tensor cores                     */
+    ISOCLUST_PATH_OMEGA_GRAM_LISTS = 3 /* the Gram from the rows' non-zeros                */
+};
+void isoclust_last_paths(int32_t *paths2);
+
 /* How the last isoclust_cluster_batched / _batched_detail call on this
  * process ran its device work: 0 launched kernel by kernel, 1 captured into
  * CUDA graphs and launched them, 2 replayed the graphs of the previous call.

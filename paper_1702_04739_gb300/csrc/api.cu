@@ -83,6 +83,7 @@ static thread_local int64_t g_prof_cnt[4] = {0, 0, 0, 0};
 static thread_local int64_t g_prof_mst_tiles[2] = {0, 0};     // tile pairs swept, and a full sweep's
 static thread_local unsigned long long g_prof_tiles[4] = {0, 0, 0, 0};
 static thread_local int g_prof_sym = 0;
+static thread_local int32_t g_prof_paths[2] = {0, 0};         // isoclust_last_paths
 static thread_local double g_prof_omega_kernel_ms = 0.0;
 static thread_local double g_prof_omega_gram_ms = 0.0;
 static thread_local int64_t g_prof_omega_gram_blocks = 0;
@@ -738,6 +739,14 @@ static isoclust_status cluster_impl(const void *X, int64_t n, int32_t d, int32_t
     memset(g_prof_tiles, 0, sizeof(g_prof_tiles));
     if (permuted) ISO_CUDA(cudaMemcpy(g_prof_tiles, P.tiles, sizeof(g_prof_tiles), cudaMemcpyDeviceToHost));
     g_prof_sym = symmetric ? (gram ? 3 : (use_tc ? 2 : 1)) : 0;
+    g_prof_paths[0] = sp_mst      ? ISOCLUST_PATH_TREE_LISTS
+                      : dist_used ? ISOCLUST_PATH_TREE_STORED
+                      : tc_used   ? ISOCLUST_PATH_TREE_TC_SWEEP
+                                  : ISOCLUST_PATH_TREE_SWEEP;
+    g_prof_paths[1] = !need_labels || o.omega_mode != ISOCLUST_OMEGA_FULL ? ISOCLUST_PATH_OMEGA_NONE
+                      : !gram                                            ? ISOCLUST_PATH_OMEGA_SUMS
+                      : sp_mst                                           ? ISOCLUST_PATH_OMEGA_GRAM_LISTS
+                                                                         : ISOCLUST_PATH_OMEGA_GRAM_TC;
     g_prof_omega_kernel_ms = symmetric ? ev.ms(8, 9) : 0.0;
     g_prof_omega_gram_ms = (symmetric && gram) ? g_prof_omega_kernel_ms : 0.0;
     g_prof_omega_gram_blocks = (symmetric && gram) ? (int64_t)g_prof_tiles[3] : 0;
@@ -1140,6 +1149,8 @@ static isoclust_status cluster_sets_impl(const void *X, const int64_t *offsets, 
     g_prof_cnt[3] = 0;
     ISO_CUDA(cudaMemcpy(g_prof_tiles, B.tiles, sizeof(g_prof_tiles), cudaMemcpyDeviceToHost));
     g_prof_sym = gram ? 3 : 1;
+    g_prof_paths[0] = ISOCLUST_PATH_TREE_TC_SWEEP;
+    g_prof_paths[1] = gram ? ISOCLUST_PATH_OMEGA_GRAM_TC : ISOCLUST_PATH_OMEGA_SUMS;
     g_prof_omega_kernel_ms = nitems > 0 ? E.ms(8, 9) : 0.0;
     g_prof_omega_gram_ms = gram ? g_prof_omega_kernel_ms : 0.0;
     g_prof_omega_gram_blocks = gram ? (int64_t)g_prof_tiles[3] : 0;
@@ -1188,6 +1199,13 @@ void isoclust_last_mst_tiles(int64_t *tiles2) {
     if (tiles2) {
         tiles2[0] = g_prof_mst_tiles[0];
         tiles2[1] = g_prof_mst_tiles[1];
+    }
+}
+
+void isoclust_last_paths(int32_t *paths2) {
+    if (paths2) {
+        paths2[0] = g_prof_paths[0];
+        paths2[1] = g_prof_paths[1];
     }
 }
 

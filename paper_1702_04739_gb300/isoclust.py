@@ -121,6 +121,8 @@ def load(build_if_missing: bool = True):
         lib.isoclust_set_mst_prune.argtypes = [ctypes.c_int32]
         lib.isoclust_set_test_stalled_wait.restype = ctypes.c_int
         lib.isoclust_set_test_stalled_wait.argtypes = [ctypes.c_int32]
+        lib.isoclust_last_paths.restype = None
+        lib.isoclust_last_paths.argtypes = [_P]
         lib.isoclust_last_mst_tiles.restype = None
         lib.isoclust_last_mst_tiles.argtypes = [_P]
         lib.isoclust_last_omega_tiles.restype = None
@@ -472,11 +474,15 @@ def last_profile() -> dict:
     lib.isoclust_last_omega_tiles(tl)
     mt = (ctypes.c_int64 * 2)()
     lib.isoclust_last_mst_tiles(mt)
+    paths = (ctypes.c_int32 * 2)()
+    lib.isoclust_last_paths(paths)
     gb, gf = ctypes.c_int64(0), ctypes.c_int64(0)
     gms = float(lib.isoclust_last_omega_gram_ms(ctypes.byref(gb), ctypes.byref(gf)))
     return dict(omega_tiles=tl[0], omega_tiles_dw=tl[1], omega_symmetric=tl[2],
                 omega_kernel_ms=float(lib.isoclust_last_omega_kernel_ms()),
                 omega_gram_ms=gms, omega_gram_blocks=int(gb.value), omega_gram_direct_pairs=int(gf.value),
+                tree_path=("sweep", "tc_sweep", "stored", "lists")[paths[0]],
+                omega_path=("none", "sums", "gram_tc", "gram_lists")[paths[1]],
                 mst_tiles_swept=mt[0], mst_tiles_full=mt[1], validate_ms=t[0], weights_ms=t[1], mst_ms=t[2], orient_ms=t[3], search_ms=t[4], labels_ms=t[5],
                 boruvka_rounds=c[0], rescanned_rows=c[1], alg1_passes=c[2], tree_depth=c[3])
 
