@@ -40,13 +40,13 @@ __device__ __forceinline__ void dw_add(float &h, float &l, float bh, float bl) {
     fast_two_sum(s, e, h, l);
 }
 
-// (a - b)^2 as a double-word.  A difference's rounding error enters with its
-// square too: without it every squared difference is 2^-50 too small on average.
+// (a - b)^2 as a double-word (the square of the difference's own rounding, 2^-50
+// of it at most on average, is left out)
 __device__ __forceinline__ void dw_square_diff(float a, float b, float &p, float &q) {
     float s, e;
     two_sum(a, -b, s, e);
     p = __fmul_rn(s, s);
-    q = __fmaf_rn(e, e, __fmaf_rn(__fadd_rn(s, s), e, __fmaf_rn(s, s, -p)));
+    q = __fmaf_rn(__fadd_rn(s, s), e, __fmaf_rn(s, s, -p));
 }
 
 // exp(-z) * 1 for z given as a double-word, result as a double-word.
