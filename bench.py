@@ -243,9 +243,9 @@ def omega_roofline(torch, dev, prof, n_pairs_alg, d, workload, sets=False):
 
 
 def omega_fused_roofline(prof, peaks, src, alu_peak, sms, kernel_ms, items, d, alg_flop):
-    """omega with the Gram on the tensor cores, one kernel: ALU-bound for rows
-    of up to about 1,000 dimensions, tensor-bound beyond.  FP32-pipe
-    instructions of the algorithm as built: 147 per pair of a kept 64 x 64
+    """omega with the Gram on the tensor cores, one kernel: bound by FP32 issue
+    for rows of a few hundred dimensions, by the reads of the rows in longer
+    ones.  FP32-pipe instructions of the algorithm as built: 147 per pair of a kept 64 x 64
     tile pair (fold of the accumulators 28, d2 and its test 27, root 12, shift
     15, double-word exp 48, the two sums 17) and 18.75 d + 95 per pair that took
     the direct sum; MMAs as issued: 34 digit-plane products of

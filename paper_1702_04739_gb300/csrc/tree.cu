@@ -1113,10 +1113,11 @@ __global__ void __launch_bounds__(1024) k_cand_select(SearchState *S, uint32_t *
 // Algorithm 1 on the whole tree out of shared memory, level by level from the
 // deepest, in BFS order (a vertex's children are then contiguous).  A level
 // costs a barrier and a few shared-memory round trips where a
-// step of the walks through global memory costs 2.5 us: 4,898 points (depth
-// 116) 0.28 ms a pass -> 0.04.  The block that finishes last updates the
-// search and picks the next thresholds, so a pass is one launch.  States go
-// out by [threshold][BFS position].
+// step of the walks through global memory costs 2.5 us: the search of 4,898
+// points (depth 116) 3.97 ms in 14 passes -> 1.0 in 5, 1.7 us a level (a vertex
+// with many children adds them one after another).  The block that finishes
+// last updates the search and picks the next thresholds, so a pass is one
+// launch.  States go out by [threshold][BFS position].
 constexpr int SM_THREADS = 512, SM_AHEAD = 4, SM_LEVELS = 1024;
 constexpr int SM_MAX_N = 12288;       // 17 bytes a vertex: 204 KB of shared memory
 constexpr int SM_MIN_SMEM = 2 * CAND_BUCKETS * (int)sizeof(uint32_t);
